@@ -168,17 +168,17 @@ typedef struct aw_tune {
  * the call forks from and joins back into the caller's stream, also inside
  * the graph of aw_grid_batched).  The TILES kernel is bound by the L2->SM
  * stream of kernel values, the OFFSETS kernel by its atomics, so sharing the
- * SMs between them beats either alone.  REGION: work items of one bin and
- * one grid tile whose side is chosen per support, sorted by oversampled
- * offset; the CTA accumulates the tile's output region (tile + support - 1
- * cells square, at most 56) in shared memory, each thread holding kernel
- * taps in registers for all visibilities of an offset (full-pol: one tap's 16
- * Mueller values; Stokes I: up to 18 taps of one value), and adds the region to
- * the grid once; bins of planes from split_planes on, and bins whose support
- * has no region form (above 49 cells; full-pol: rows that do not split into
- * passes of 32 taps over 4-10 warps; Stokes I: not a multiple of 4), take
- * OFFSETS on the plan's second stream at the same time.  All modes give the
- * same grid up to FP32 rounding order. */
+ * SMs between them beats either alone.  REGION: tasks of one bin, one grid
+ * tile and one footprint block, sorted by oversampled offset; a CTA
+ * accumulates one plane of the tile's output region (56 cells square) in
+ * shared memory, each thread holding kernel taps in registers for all
+ * visibilities of an offset, and adds the region to the grid once; bins whose
+ * support has no region form (padded to a multiple of 8 taps a side it would
+ * cost more than 1.8 times the taps; Stokes I: above 48 cells) take OFFSETS on
+ * the plan's second stream at the same time.  split_planes is checked (0..nw)
+ * but does not move planes to OFFSETS, which is the slower one at every
+ * support with a region form.  All modes give the same grid up to FP32
+ * rounding order. */
 enum { AW_GRID_TILES = 0, AW_GRID_OFFSETS = 1, AW_GRID_HYBRID = 2, AW_GRID_REGION = 3 };
 
 typedef struct aw_plan_info {
@@ -192,7 +192,7 @@ typedef struct aw_plan_info {
     double mean_taps;        /* mean S^2 over the valid visibilities              */
     int64_t nitems_degrid;   /* degridding work items                             */
     int32_t grid_kernels;    /* kernels one aw_grid / aw_grid_batched call launches */
-    int32_t region_lists;    /* AW_GRID_REGION: supports on the region kernel      */
+    int32_t region_lists;    /* AW_GRID_REGION: task lists of the region kernel    */
 } aw_plan_info;
 
 typedef struct aw_stats {

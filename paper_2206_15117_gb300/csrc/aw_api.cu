@@ -234,8 +234,7 @@ static void free_plan(aw_plan *p) {
     if (p->d_items_ht) aw_dev_free(p->d_items_ht);
     if (p->d_items_ho) aw_dev_free(p->d_items_ho);
     if (p->d_rec_rg) aw_dev_free(p->d_rec_rg);
-    for (auto &c : p->rclasses)
-        if (c.d_items) aw_dev_free(c.d_items);
+    if (p->d_items_rg) aw_dev_free(p->d_items_rg);
     if (p->d_rcounter) aw_dev_free(p->d_rcounter);
     if (p->ev_fork) cudaEventDestroy(p->ev_fork);
     if (p->ev_join) cudaEventDestroy(p->ev_join);
@@ -283,8 +282,7 @@ int aw_plan_query(const aw_plan *p, aw_plan_info *info) {
     info->chunk = p->tune.chunk;
     info->mean_taps = p->mean_taps;
     info->nitems_degrid = p->nitems_dg;
-    int nl = 0;
-    for (const auto &c : p->rclasses) nl += c.n > 0;
+    const int nl = p->nitems_rg > 0;
     info->region_lists = nl;
     switch (p->tune.grid_mode) {
         case AW_GRID_HYBRID: info->grid_kernels = (p->nitems_ht > 0) + (p->nitems_ho > 0); break;
@@ -356,10 +354,9 @@ static int launch_planned(aw_ctx *ctx, const aw_plan *p, const aw_kernel_set *k,
         return (int)std::max<int64_t>(c, 1);
     };
     if (p->tune.grid_mode == AW_GRID_REGION) {
-        // the region lists on the caller's stream; the bins that take no region
-        // (wide supports, or planes from split_planes on) with the OFFSETS
-        // kernel on the second stream at the same time, one CTA per SM (it
-        // fits beside two region CTAs: registers, shared memory, threads)
+        // the region tasks on the caller's stream; the bins that take no region
+        // with the OFFSETS kernel on the second stream at the same time, one CTA
+        // per SM (it fits beside the region CTAs in registers and threads)
         if (p->nitems_ho == 0) return aw_launch_grid_region(p, k, vis, weight, grid, s);
         if (p->nreg == 0) {   // no bin takes a region: OFFSETS alone, every SM
             aw_grid_launch Lo{p, k, vis, weight, grid, false, 0, s, AW_GRID_OFFSETS, p->d_items_ho, p->nitems_ho};
@@ -553,27 +550,20 @@ int aw_autotune(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *k, aw_
         if (rc) break;
         if (ms_best < best) { best = ms_best; bt = tu; }
     }
-    // the region schedule: the w planes up to the last one whose support is at
-    // most 32, 40 or 48 cells on the region kernel (bins whose support has no
-    // region form stay on OFFSETS), the rest on OFFSETS at the same time (its
-    // super-tile the larger one)
-    if (!rc) {
-        int last_split = -1;
-        for (int lim : {32, 40, 48}) {
-            int q = 0;
-            while (q < k->spec.nw && k->supports[(size_t)q] <= lim) ++q;
-            if (q == 0 || q == last_split) continue;
-            last_split = q;
-            aw_tune tu{bt.tile, bt.chunk, 2, 1024, AW_GRID_REGION, q};
-            aw_plan *p = new aw_plan();
-            p->device = ctx->device;
-            int r2 = aw_plan_build(ctx, vis, k, &tu, p, s);
-            float ms_best = 1e30f;
-            if (!r2) r2 = time_plan(p, &ms_best);
-            free_plan(p);
-            if (!r2 && ms_best < best) { best = ms_best; bt = tu; }
-            if (r2) cudaGetLastError();   // a candidate that cannot be built is skipped
-        }
+    // the region schedule (bins whose support has no region form stay on
+    // OFFSETS, its super-tile the larger one)
+    bool any_region = false;
+    for (int32_t S : k->bin_support) any_region = any_region || aw_rg_eligible(S, k->spec.npol);
+    if (!rc && any_region) {
+        aw_tune tu{bt.tile, bt.chunk, 2, 1024, AW_GRID_REGION, k->spec.nw};
+        aw_plan *p = new aw_plan();
+        p->device = ctx->device;
+        int r2 = aw_plan_build(ctx, vis, k, &tu, p, s);
+        float ms_best = 1e30f;
+        if (!r2) r2 = time_plan(p, &ms_best);
+        free_plan(p);
+        if (!r2 && ms_best < best) { best = ms_best; bt = tu; }
+        if (r2) cudaGetLastError();   // a candidate that cannot be built is skipped
     }
     // the hybrid schedule: the first planes holding about a quarter to a half
     // of the visibility-taps on TILES, the rest on OFFSETS, at 2 or 3 TILES CTAs

@@ -145,20 +145,16 @@ struct aw_plan {
     int64_t nitems_ho = 0;
     cudaStream_t aux = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    // AW_GRID_REGION: the valid visibilities of the bins whose support fits a
-    // shared-memory region, by (bin, region tile, oversampled offset,
-    // position), cut into items {start, count, bin, tile}; one item list per
-    // support (each launched with its own CTA size).  The other bins' degridding
-    // items (d_items_ho) take the OFFSETS schedule on the second stream.
+    // AW_GRID_REGION: the valid visibilities of the bins on the region kernels,
+    // by (bin, region tile, oversampled offset, position), cut into tasks
+    // {start, count, bin, aw_rg_pack(tile, footprint block)}.  The other bins'
+    // degridding items (d_items_ho) take the OFFSETS schedule on the second
+    // stream.
     aw_rec *d_rec_rg = nullptr;
     int64_t nreg = 0;
-    struct RegionClass {
-        int S = 0, T = 0, BT = 0;
-        int4 *d_items = nullptr;
-        int64_t n = 0;
-    };
-    std::vector<RegionClass> rclasses;
-    unsigned int *d_rcounter = nullptr;   // [AW_RG_MAXCLASS] work-queue heads
+    int4 *d_items_rg = nullptr;
+    int64_t nitems_rg = 0;
+    unsigned int *d_rcounter = nullptr;   // work-queue heads of the region kernels
     // coordinate inputs kept for aw_plan_coords
     aw_vis_desc vis{};
     double uscale = 0, half = 0, winv = 0;
@@ -180,14 +176,45 @@ struct aw_plan {
     }
 };
 
-// REGION gridding: largest region side (cells) held in shared memory, and the
-// most distinct supports (item lists) a plan launches.
-#ifndef AW_RG_RMAX_CELLS
-#define AW_RG_RMAX_CELLS 56
-#endif
-constexpr int AW_RG_RMAX = AW_RG_RMAX_CELLS;
-constexpr int AW_RG_MAXCLASS = 64;
-constexpr int AW_RG_MAXV = 1024;   // visibilities per region work item
+// ---------------------------------------------------------------- regions
+// REGION schedule: a CTA accumulates one plane of a grid region of AW_RG_R x
+// AW_RG_R cells in shared memory.  A footprint of S x S taps is cut along each
+// axis into blocks of 24 or 16 taps (one of 8 for S <= 8; the last block may
+// reach past the footprint, its absent taps have kernel value 0), and a task
+// is one block of the footprints that start in one T x T grid tile, T + block
+// - 1 <= AW_RG_R.
+constexpr int AW_RG_R = 56;
+constexpr int AW_RG_MAXV = 1024;      // visibilities per gridding task
+constexpr int AW_RG_COUNTERS = 4;
+
+// blocks along an axis: n24 of 24 taps, then n16 of 16 (S <= 8: one of 8)
+__host__ __device__ inline int aw_rg_n24(int S) {
+    const int k = (S + 7) / 8;
+    return k <= 1 ? 0 : (k - (k % 3 == 0 ? 0 : k % 3 == 2 ? 2 : 4)) / 3;
+}
+__host__ __device__ inline int aw_rg_nblk(int S) {
+    const int k = (S + 7) / 8;
+    return k <= 1 ? 1 : aw_rg_n24(S) + (k % 3 == 0 ? 0 : k % 3 == 2 ? 1 : 2);
+}
+__host__ __device__ inline int aw_rg_blk_width(int S, int i) { return S <= 8 ? 8 : i < aw_rg_n24(S) ? 24 : 16; }
+__host__ __device__ inline int aw_rg_blk_first(int S, int i) {
+    const int a = aw_rg_n24(S);
+    return i <= a ? 24 * i : 24 * a + 16 * (i - a);
+}
+__host__ __device__ inline int aw_rg_tile(int S) {
+    return AW_RG_R + 1 - (S <= 8 ? 8 : aw_rg_n24(S) ? 24 : 16);
+}
+// Supports on the region kernels: padding the footprint to a multiple of 8 taps
+// a side costs at most 1.8 times the taps (about what OFFSETS costs more).
+// Stokes I: up to 48 cells (wider ones hold few visibilities a tile).
+inline bool aw_rg_eligible(int S, int npol) {
+    const int p = (S + 7) / 8 * 8;
+    return S >= 2 && S <= (npol == 1 ? 48 : 128) && 10 * p * p <= 18 * S * S;
+}
+// task word: tile column and row (9 bits each: at most 16384 / 33), block column and row (3 bits each)
+__host__ __device__ inline int aw_rg_pack(int tx, int ty, int bx, int by) {
+    return tx | ty << 9 | bx << 18 | by << 21;
+}
 
 // Visibilities per degridding work item: 8 warps x 4 visibilities.
 constexpr int AW_DG_VB = 4;
@@ -237,12 +264,7 @@ struct aw_grid_launch {
     int64_t nitems = 0;
 };
 int aw_launch_grid(const aw_grid_launch &L);
-// REGION schedule (aw_grid_region.cu): region tile side for support S (0: the
-// support does not fit a region), CTA size for support S, and the launch of
-// every support's item list on stream s.
-int aw_region_tile(int S, int npol);
-int aw_region_rows(int S);
-int aw_region_threads(int S, int npol);
+// REGION schedule (aw_grid_region.cu): the gridding tasks of a plan on stream s.
 int aw_launch_grid_region(const aw_plan *p, const aw_kernel_set *k, const void *vis, const float *weight, void *grid,
                           cudaStream_t s);
 int aw_region_bounds_status(unsigned int *v, int reset);

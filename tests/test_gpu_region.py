@@ -1,0 +1,66 @@
+"""GPU: the region gridding kernel at the edges of its forms (footprint blocks
+of 8, 16 and 24 taps and their mixtures, supports padded to a multiple of 8,
+runs and tasks longer than a staging round) against the FP64 oracle."""
+import math
+
+import numpy as np
+import pytest
+
+from paper_2206_15117_gb300 import synthetic as sy
+from tests.gpu_cases import case_fullpol, rel_err
+from tests.test_gpu_grid import Case, _check_degrid, _check_grid
+
+pytestmark = pytest.mark.gpu
+
+REGION = 3
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_2206_15117_gb300 import aw
+    return aw.aw_create(0)
+
+
+def _stokes_i(supports, n_t=60, radius=120.0, N=256):
+    ob = sy.small_observation(n_ant=14, radius_m=radius, n_t=n_t, freq=(1.2e9, 1.35e9, 1.5e9), seed=sy.BASE_SEED + 410)
+    return ob, dict(N=N, dl=math.radians(3.0) / N, OS=8, W=7.0, npol=1, nw=len(supports), w_max=ob.w_max,
+                    supports=list(supports))
+
+
+@pytest.mark.parametrize("supports", [(7, 8, 12), (15, 16, 18), (20, 24, 28), (32, 40, 48), (56, 64, 72), (9, 10, 17)])
+@pytest.mark.parametrize("npol", [1, 4])
+def test_region_supports(ctx, npol, supports):
+    from paper_2206_15117_gb300 import aw
+    ob, kw = case_fullpol(supports=supports, n_t=30, radius=100.0) if npol == 4 else _stokes_i(supports)
+    flags = (np.random.default_rng(5).random(ob.nvis) < 0.05).astype(np.uint8)
+    c = Case(ctx, ob, kw, tune=aw.aw_tune(32, 256, 2, 256, REGION), flags=flags)
+    _check_grid(c)
+    _check_grid(c, batched=True)
+    _check_degrid(c)
+
+
+# runs of equal offset longer than a round of 64 and tasks longer than 1024, a
+# non-finite visibility among them
+@pytest.mark.parametrize("npol", [1, 4])
+def test_region_long_runs(ctx, npol):
+    from paper_2206_15117_gb300 import aw
+    sup = (16, 24, 40)
+    ob, kw = case_fullpol(supports=sup, n_t=400, radius=20.0) if npol == 4 else _stokes_i(sup, n_t=700, radius=20.0)
+    c = Case(ctx, ob, kw, tune=aw.aw_tune(32, 256, 2, 256, REGION))
+    co, ok = c.co, c.co.valid == 1
+    run = np.stack([co.bin[ok], co.y0[ok] // 41, co.x0[ok] // 41, co.fy[ok], co.fx[ok]])
+    assert np.unique(run, axis=1, return_counts=True)[1].max() > 64
+    c.vis[17, 0] = np.nan
+    _check_grid(c)
+    _check_degrid(c)
+
+
+@pytest.mark.parametrize("storage,tol", [(1, 4e-3), (2, 5e-4)])
+def test_region_padded_support_reduced_precision(ctx, storage, tol):
+    from paper_2206_15117_gb300 import aw
+    ob, kw = case_fullpol(supports=(12, 20, 40), n_t=30, radius=100.0)
+    c = Case(ctx, ob, kw, storage=storage, tune=aw.aw_tune(32, 256, 2, 256, REGION))
+    l2, mx = rel_err(c.gpu_grid(batched=True)[0], c.oracle_grid()[0])
+    assert l2 < tol and mx < 4 * tol, (l2, mx)
+    l2, _ = rel_err(c.gpu_degrid(), c.oracle_degrid())
+    assert l2 < tol, l2
