@@ -235,6 +235,7 @@ static void free_plan(aw_plan *p) {
     if (p->d_items_ho) aw_dev_free(p->d_items_ho);
     if (p->d_rec_rg) aw_dev_free(p->d_rec_rg);
     if (p->d_items_rg) aw_dev_free(p->d_items_rg);
+    if (p->d_items_rgd) aw_dev_free(p->d_items_rgd);
     if (p->d_rcounter) aw_dev_free(p->d_rcounter);
     if (p->ev_fork) cudaEventDestroy(p->ev_fork);
     if (p->ev_join) cudaEventDestroy(p->ev_join);

@@ -446,6 +446,7 @@ struct DegridArgs {
     const int4 *items;       // [nitems] {start, count, bin, 0} over rec_dg
     int64_t nitems;
     int64_t nvis, nvalid;
+    int64_t tail_end;        // visibilities [nvalid, tail_end) of rec predict zero here
     const void *ktab;
     const int64_t *bin_offset;
     const int32_t *bin_support;
@@ -770,7 +771,7 @@ __global__ void __launch_bounds__(256, NPOL == 1 ? 4 : 2) degrid_items_kernel(De
         }
     }
     // visibilities that were not gridded (outside or flagged) predict zero
-    for (int64_t i = a.nvalid + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.nvis;
+    for (int64_t i = a.nvalid + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.tail_end;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t o = (int64_t)a.rec[i].orig * NPOL;
 #pragma unroll
@@ -957,6 +958,15 @@ int aw_launch_degrid(const aw_plan *p, const aw_kernel_set *k, const void *grid,
     a.nitems = p->nitems_dg;
     a.nvis = p->nvis;
     a.nvalid = p->nvalid;
+    a.tail_end = p->nvis;
+    if (p->nitems_rgd > 0) {
+        // region tasks (and the visibilities not gridded) first, the other bins here
+        const int rc = aw_launch_degrid_region(p, k, grid, vis_out, s, sub_from);
+        if (rc || p->nitems_ho == 0) return rc;
+        a.items = p->d_items_ho;
+        a.nitems = p->nitems_ho;
+        a.tail_end = p->nvalid;
+    }
     a.ktab = k->d_table;
     a.bin_offset = k->d_bin_offset;
     a.bin_support = k->d_bin_support;
@@ -994,7 +1004,10 @@ extern "C" int aw_debug_bounds_status(uint32_t *status, int32_t reset) {
     }
     int rc = aw_region_bounds_status(&vr, reset);
     if (rc) return rc;
-    *status = v ? v : vr;
+    unsigned int vd = 0;
+    rc = aw_degrid_region_bounds_status(&vd, reset);
+    if (rc) return rc;
+    *status = v ? v : vr ? vr : vd;
     return AW_OK;
 #else
     (void)reset;

@@ -154,6 +154,10 @@ struct aw_plan {
     int64_t nreg = 0;
     int4 *d_items_rg = nullptr;
     int64_t nitems_rg = 0;
+    // Stokes I: the region degridding tasks over the same records (all blocks of
+    // a footprint in one task)
+    int4 *d_items_rgd = nullptr;
+    int64_t nitems_rgd = 0;
     unsigned int *d_rcounter = nullptr;   // work-queue heads of the region kernels
     // coordinate inputs kept for aw_plan_coords
     aw_vis_desc vis{};
@@ -185,6 +189,7 @@ struct aw_plan {
 // - 1 <= AW_RG_R.
 constexpr int AW_RG_R = 56;
 constexpr int AW_RG_MAXV = 1024;      // visibilities per gridding task
+constexpr int AW_RG_MAXV_DG = 256;   // visibilities per degridding task
 constexpr int AW_RG_COUNTERS = 4;
 
 // blocks along an axis: n24 of 24 taps, then n16 of 16 (S <= 8: one of 8)
@@ -268,6 +273,11 @@ int aw_launch_grid(const aw_grid_launch &L);
 int aw_launch_grid_region(const aw_plan *p, const aw_kernel_set *k, const void *vis, const float *weight, void *grid,
                           cudaStream_t s);
 int aw_region_bounds_status(unsigned int *v, int reset);
+// Region degridding (aw_degrid_region.cu) of the plan's region tasks, and zero
+// (or sub_from) for the visibilities that are not gridded.
+int aw_launch_degrid_region(const aw_plan *p, const aw_kernel_set *k, const void *grid, void *vis_out,
+                            cudaStream_t s, const void *sub_from);
+int aw_degrid_region_bounds_status(unsigned int *v, int reset);
 // cum[q] = share of the plan's visibility-taps (sum of S^2) in w planes < q, q = 0..nw
 int aw_plan_plane_taps(const aw_plan *plan, std::vector<double> &cum, cudaStream_t s);
 int aw_launch_degrid(const aw_plan *plan, const aw_kernel_set *kset, const void *grid,

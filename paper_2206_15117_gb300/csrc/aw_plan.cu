@@ -481,27 +481,17 @@ int build_items(const uint64_t *keys, int64_t nv, int shift, int chunk, const aw
     return AW_OK;
 }
 
-// The region tasks of the nreg records `rec` with sorted keys `keys` (segments
-// of equal key >> shift) under the per-bin geometry geo; allocates *tasks.
-int build_region_tasks(const uint64_t *keys, int64_t nreg, int shift, const aw_rec *rec, const int4 *geo,
-                       uint32_t *flag, uint32_t *segid, void *scratch, int4 **tasks, int64_t *ntasks,
-                       cudaStream_t s) {
-    DevBuf bstarts, bcnt, bbase;
-    int64_t nseg = 0;
-    int rc = build_segments(keys, nreg, shift, flag, segid, scratch, bstarts, &nseg, s);
-    if (rc) return rc;
-    AW_CUDA_TRY(aw_dev_malloc(&bcnt.p, sizeof(uint32_t) * nseg));
-    AW_CUDA_TRY(aw_dev_malloc(&bbase.p, sizeof(uint32_t) * nseg));
-    rg_count_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>((uint32_t *)bstarts.p, nseg, (uint32_t)nreg, rec, geo,
-                                                          (uint32_t *)bcnt.p);
+// The region tasks of the segments `starts` of the nreg records `rec` under the
+// per-bin geometry geo; allocates *tasks.  `cnt` and `base` hold nseg words each.
+int build_region_tasks(const uint32_t *starts, int64_t nseg, int64_t nreg, const aw_rec *rec, const int4 *geo,
+                       uint32_t *cnt, uint32_t *base, void *scratch, int4 **tasks, int64_t *ntasks, cudaStream_t s) {
+    rg_count_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>(starts, nseg, (uint32_t)nreg, rec, geo, cnt);
     AW_CHECK_LAUNCH();
-    rc = scan_counts((uint32_t *)bcnt.p, (uint32_t *)bbase.p, nseg, scratch, ntasks, s);
+    const int rc = scan_counts(cnt, base, nseg, scratch, ntasks, s);
     if (rc) return rc;
     AW_CUDA_TRY(aw_dev_malloc(tasks, sizeof(int4) * std::max<int64_t>(*ntasks, 1)));
-    rg_emit_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>((uint32_t *)bstarts.p, (uint32_t *)bbase.p, nseg,
-                                                         (uint32_t)nreg, rec, geo, *tasks);
+    rg_emit_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>(starts, base, nseg, (uint32_t)nreg, rec, geo, *tasks);
     AW_CHECK_LAUNCH();
-    AW_CUDA_TRY(cudaStreamSynchronize(s));
     return AW_OK;
 }
 
@@ -547,18 +537,21 @@ static int build_region(aw_plan *plan, const aw_kernel_set *ks, int64_t nv, uint
                         uint64_t *k1, uint32_t *v1, uint32_t *counts, uint32_t *offs, void *scratch,
                         cudaStream_t s) {
     const int nb = ks->nbins;
-    std::vector<int4> geo((size_t)nb, make_int4(0, 0, 0, 0));
+    // gridding geometry of every bin, then the degridding one
+    std::vector<int4> geo((size_t)nb * 2, make_int4(0, 0, 0, 0));
     bool all = true;
     for (int b = 0; b < nb; ++b) {
         const int S = ks->bin_support[(size_t)b];
-        if (aw_rg_eligible(S, plan->npol))
+        if (aw_rg_eligible(S, plan->npol)) {
             geo[(size_t)b] = make_int4(aw_rg_tile(S), AW_RG_MAXV, aw_rg_nblk(S), 0);
-        else
+            geo[(size_t)nb + b] = make_int4(aw_rg_tile(S), AW_RG_MAXV_DG, 1, 0);
+        } else {
             all = false;
+        }
     }
     DevBuf dgeo, dcnt;
-    AW_CUDA_TRY(aw_dev_malloc(&dgeo.p, sizeof(int4) * std::max(nb, 1)));
-    AW_CUDA_TRY(cudaMemcpyAsync(dgeo.p, geo.data(), sizeof(int4) * nb, cudaMemcpyHostToDevice, s));
+    AW_CUDA_TRY(aw_dev_malloc(&dgeo.p, sizeof(int4) * geo.size()));
+    AW_CUDA_TRY(cudaMemcpyAsync(dgeo.p, geo.data(), sizeof(int4) * geo.size(), cudaMemcpyHostToDevice, s));
     const int4 *d_geo = (const int4 *)dgeo.p;
     AW_CUDA_TRY(aw_dev_malloc(&dcnt.p, sizeof(unsigned long long)));
     AW_CUDA_TRY(cudaMemsetAsync(dcnt.p, 0, sizeof(unsigned long long), s));
@@ -585,9 +578,24 @@ static int build_region(aw_plan *plan, const aw_kernel_set *ks, int64_t nv, uint
     if (plan->nreg > 0) {
         gather_rec_kernel<<<grid_blocks(plan->nreg, 256), 256, 0, s>>>(plan->d_rec, v0, plan->nreg, plan->d_rec_rg);
         AW_CHECK_LAUNCH();
-        rc = build_region_tasks(k0, plan->nreg, osb + 12, plan->d_rec_rg, d_geo, counts, offs, scratch,
+        DevBuf bstarts, bcnt, bbase;
+        int64_t nseg = 0;
+        rc = build_segments(k0, plan->nreg, osb + 12, counts, offs, scratch, bstarts, &nseg, s);
+        if (rc) return rc;
+        AW_CUDA_TRY(aw_dev_malloc(&bcnt.p, sizeof(uint32_t) * nseg));
+        AW_CUDA_TRY(aw_dev_malloc(&bbase.p, sizeof(uint32_t) * nseg));
+        const uint32_t *starts = (const uint32_t *)bstarts.p;
+        uint32_t *cnt = (uint32_t *)bcnt.p, *base = (uint32_t *)bbase.p;
+        rc = build_region_tasks(starts, nseg, plan->nreg, plan->d_rec_rg, d_geo, cnt, base, scratch,
                                 &plan->d_items_rg, &plan->nitems_rg, s);
         if (rc) return rc;
+        if (plan->npol == 1) {
+            rc = build_region_tasks(starts, nseg, plan->nreg, plan->d_rec_rg, d_geo + nb, cnt, base, scratch,
+                                    &plan->d_items_rgd, &plan->nitems_rgd, s);
+            if (rc) return rc;
+        }
+        // the temporaries are freed here: finish the kernels that read them
+        AW_CUDA_TRY(cudaStreamSynchronize(s));
     }
     // the other bins: their degridding items on the OFFSETS schedule
     if (!all) {
