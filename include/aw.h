@@ -382,7 +382,8 @@ int aw_autotune(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *kset, 
  *
  * real part, c(q) = psi(2 l_q / F) the taper (grid correction); row/column 0
  * are written as 0.  grid (device complex64 [npol][N][N], kset's N and npol)
- * is used as FFT scratch and left transformed; image: device float
+ * is used as FFT scratch and left transformed (the plain unscaled inverse FFT);
+ * image: device float
  * [npol][N][N].  cuFFT (FP32 complex) plus the library's own shift and
  * grid-correction kernels.
  */
