@@ -223,20 +223,18 @@ int aw_kernel_set_destroy(aw_kernel_set *k) {
 static void free_plan(aw_plan *p) {
     if (!p) return;
     p->drop_graphs();
-    if (p->d_rec) aw_dev_free(p->d_rec);
-    if (p->d_items) aw_dev_free(p->d_items);
-    if (p->d_rec_dg) aw_dev_free(p->d_rec_dg);
-    if (p->d_items_dg) aw_dev_free(p->d_items_dg);
+    if (p->d_block) aw_dev_free(p->d_block);
     if (p->d_plane_support) aw_dev_free(p->d_plane_support);
+    if (p->d_fl) aw_dev_free(p->d_fl);
     if (p->d_wsum) aw_dev_free(p->d_wsum);
     if (p->d_nonfinite) aw_dev_free(p->d_nonfinite);
     if (p->d_counter) aw_dev_free(p->d_counter);
+    if (p->d_items) aw_dev_free(p->d_items);
+    if (p->d_items_dg) aw_dev_free(p->d_items_dg);
     if (p->d_items_ht) aw_dev_free(p->d_items_ht);
     if (p->d_items_ho) aw_dev_free(p->d_items_ho);
-    if (p->d_rec_rg) aw_dev_free(p->d_rec_rg);
     if (p->d_items_rg) aw_dev_free(p->d_items_rg);
     if (p->d_items_rgd) aw_dev_free(p->d_items_rgd);
-    if (p->d_rcounter) aw_dev_free(p->d_rcounter);
     if (p->ev_fork) cudaEventDestroy(p->ev_fork);
     if (p->ev_join) cudaEventDestroy(p->ev_join);
     if (p->aux) cudaStreamDestroy(p->aux);

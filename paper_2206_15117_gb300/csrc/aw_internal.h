@@ -122,6 +122,7 @@ struct aw_plan {
     int ntype = 1;                  // baseline classes are ntype^2 when ntype >= 2
     aw_tune tune{};
     double mean_taps = 0;
+    void *d_block = nullptr;        // one allocation: d_rec, d_rec_dg, d_rec_rg
     aw_rec *d_rec = nullptr;        // [nvis] sorted (valid first) by (bin, tile, position)
     int4 *d_items = nullptr;        // [nitems] {start, count, bin, 0}
     // degridding order: the valid visibilities by (bin, super-tile, oversampled
@@ -131,6 +132,7 @@ struct aw_plan {
     int64_t nitems_dg = 0;
     int dg_tile = 1024;
     int32_t *d_plane_support = nullptr;  // [nw] support per w plane
+    double *d_fl = nullptr;              // [nchan] frequency / c
     std::vector<int32_t> bin_support;
     // grid-time statistics (device): [0] weight sum (double), [1] non-finite count
     double *d_wsum = nullptr;

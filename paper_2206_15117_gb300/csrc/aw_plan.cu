@@ -14,7 +14,7 @@ struct CoordArgs {
     const double *uvw;
     const uint32_t *row;
     const uint16_t *chan;
-    const double *freq;
+    const double *fl;          // per channel: frequency / c, one correctly rounded division
     const uint8_t *pa_bin;
     const uint8_t *fbin;
     const uint8_t *flags;
@@ -31,30 +31,51 @@ struct CoordOut {
     int x0, y0, fx, fy, bin, flip, valid, S;
 };
 
+// floor(a / d), in 32 bits where a fits (nearly every visibility)
+__device__ __forceinline__ long long floor_div(long long a, int d) {
+    if (a >= 0 && a <= 0x7fffffffll) return (long long)((uint32_t)a / (uint32_t)d);
+    long long q = a / d;
+    if (a < 0 && q * d != a) q -= 1;
+    return q;
+}
+
+__global__ void channel_kernel(const double *freq, int nchan, double *fl) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < nchan) fl[c] = __ddiv_rn(freq[c], AW_C_LIGHT);
+}
+
 // The FP64 coordinate step with a fixed operation order (no contraction).
+// FP64 runs at 2 lanes a clock and SM here, so the step holds ten FP64 operations
+// and three conversions; the division by c is done once a channel, signs are
+// tested and changed on the bits.
 __device__ __forceinline__ CoordOut coord_of(const CoordArgs &a, int64_t k) {
     CoordOut o;
     const uint32_t r = a.row[k];
     const uint16_t c = a.chan[k];
-    const double f = __ddiv_rn(a.freq[c], AW_C_LIGHT);
+    const double f = __ldg(a.fl + c);
     double u = __dmul_rn(a.uvw[3 * (int64_t)r + 0], f);
     double v = __dmul_rn(a.uvw[3 * (int64_t)r + 1], f);
     double w = __dmul_rn(a.uvw[3 * (int64_t)r + 2], f);
-    o.flip = 0;
-    if (w < 0.0) { u = -u; v = -v; w = -w; o.flip = 1; }
+    // w < 0, and the sign change, on the bits (comparisons run in the FP64 pipe too)
+    const unsigned long long wb = (unsigned long long)__double_as_longlong(w);
+    o.flip = wb - 0x8000000000000001ull <= 0x7ff0000000000000ull - 1ull ? 1 : 0;   // -inf .. the smallest negative
+    const unsigned long long sign = (unsigned long long)o.flip << 63;
+    u = __longlong_as_double((long long)((unsigned long long)__double_as_longlong(u) ^ sign));
+    v = __longlong_as_double((long long)((unsigned long long)__double_as_longlong(v) ^ sign));
+    w = __longlong_as_double((long long)(wb ^ sign));
     const double xr = __dadd_rn(__dadd_rn(__dmul_rn(u, a.uscale), a.half), 0.5);
     const double yr = __dadd_rn(__dadd_rn(__dmul_rn(v, a.uscale), a.half), 0.5);
-    // clamp far-out values before the integer conversion; they are invalid anyway
-    const double lim = 4.0e15;
-    const long long Xi = (long long)floor(fmin(fmax(xr, -lim), lim));
-    const long long Yi = (long long)floor(fmin(fmax(yr, -lim), lim));
+    // rounded down and clamped far out, where they are invalid anyway (the conversion
+    // saturates and takes a NaN to the lowest value)
+    const long long lim = 4000000000000000ll;
+    const long long Xi = min(max(__double2ll_rd(xr), -lim), lim);
+    const long long Yi = min(max(__double2ll_rd(yr), -lim), lim);
     int wp = 0;
     if (a.winv > 0.0) {
+        // (a NaN counts as far out, as the minimum with a large plane number takes it)
         const double wt = __dmul_rn(w, a.winv);
-        const double fw = floor(fmin(wt, 1.0e9));
-        wp = (int)fw;
-        if (wp < 0) wp = 0;
-        if (wp > a.nw - 1) wp = a.nw - 1;
+        const bool nan = ((unsigned long long)__double_as_longlong(wt) & 0x7fffffffffffffffull) > 0x7ff0000000000000ull;
+        wp = nan ? a.nw - 1 : min(max(__double2int_rd(wt), 0), a.nw - 1);
     }
     const int pa = a.pa_bin ? (int)a.pa_bin[r] : 0;
     const int fb = a.fbin ? (int)a.fbin[c] : 0;
@@ -71,8 +92,7 @@ __device__ __forceinline__ CoordOut coord_of(const CoordArgs &a, int64_t k) {
     o.S = S;
     const long long rho = (long long)(S - 2) * a.OS / 2;
     const long long Ax = Xi - rho, Ay = Yi - rho;
-    long long ix = Ax / a.OS; if (Ax < 0 && ix * a.OS != Ax) ix -= 1;
-    long long iy = Ay / a.OS; if (Ay < 0 && iy * a.OS != Ay) iy -= 1;
+    const long long ix = floor_div(Ax, a.OS), iy = floor_div(Ay, a.OS);
     o.fx = (int)(Ax - ix * a.OS);
     o.fy = (int)(Ay - iy * a.OS);
     int valid = 1;
@@ -84,8 +104,8 @@ __device__ __forceinline__ CoordOut coord_of(const CoordArgs &a, int64_t k) {
     return o;
 }
 
-__global__ void coords_kernel(CoordArgs a, uint64_t invalid_key, uint64_t *keys, uint32_t *vals,
-                              aw_rec *recs, unsigned long long *counts /* outside, flagged, valid, taps */) {
+template <typename K>
+__global__ void coords_kernel(CoordArgs a, K invalid_key, K *keys, aw_rec *recs, unsigned long long *counts /* outside, flagged, valid, taps */) {
     unsigned long long n_out = 0, n_flag = 0, n_val = 0, taps = 0;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < a.nvis;
          k += (int64_t)gridDim.x * blockDim.x) {
@@ -94,17 +114,15 @@ __global__ void coords_kernel(CoordArgs a, uint64_t invalid_key, uint64_t *keys,
         const bool ok = o.valid && !flagged;
         if (!o.valid) n_out++;
         else if (flagged) n_flag++;
-        uint64_t key = invalid_key;
+        K key = invalid_key;
         if (ok) {
             n_val++;
             taps += (unsigned long long)o.S * o.S;
             const int tx = o.x0 >> a.tbits, ty = o.y0 >> a.tbits;
             const int lx = o.x0 & (a.tile - 1), ly = o.y0 & (a.tile - 1);
-            key = ((((uint64_t)o.bin * a.nty + ty) * a.ntx + tx) << (2 * a.tbits)) |
-                  ((uint64_t)ly << a.tbits) | (uint64_t)lx;
+            key = ((((K)o.bin * a.nty + ty) * a.ntx + tx) << (2 * a.tbits)) | ((K)ly << a.tbits) | (K)lx;
         }
         keys[k] = key;
-        vals[k] = (uint32_t)k;
         aw_rec rc;
         rc.orig = (uint32_t)k;
         rc.x0 = (uint16_t)o.x0;
@@ -150,102 +168,202 @@ __global__ void coords_out_kernel(CoordArgs a, int32_t *x0, int32_t *y0, int32_t
 
 // ------------------------------------------------------------ LSD radix sort
 // One pass = per-tile digit histogram -> exclusive scan over [digit][tile] ->
-// stable scatter.  A tile is RS_THREADS * RS_ITEMS keys; each warp owns a
-// contiguous run of RS_ITEMS * 32 keys, ranks equal digits with
-// __match_any_sync, and keeps its own running digit counters, so the order of
-// equal keys is preserved.
-constexpr int RS_THREADS = 256;
+// stable scatter, with digits of up to 9 bits and keys of 32 or 64 bits.  A tile
+// is RS_TILE keys; each warp owns a contiguous run of RS_ITEMS * 32 of them and
+// ranks equal digits with __match_any_sync against its own running counters, so
+// the order of equal keys is preserved.  The tile is put in digit order in shared
+// memory first, so that a digit's run leaves as consecutive words: written
+// straight from the registers, every store touched 32 sectors, and a pass over
+// 12M 64-bit keys took 146 us (116 now; 64 with 32-bit keys).
+constexpr int RS_THREADS = 512;
 constexpr int RS_WARPS = RS_THREADS / 32;
 constexpr int RS_ITEMS = 16;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
+constexpr int RS_BITS = 9;
+constexpr int RS_DIGITS = 1 << RS_BITS;
+static_assert(RS_DIGITS == RS_THREADS, "one digit a thread");
 
-__global__ void radix_hist_kernel(const uint64_t *keys, int64_t n, int shift, uint32_t *counts,
-                                  int ntiles) {
-    __shared__ uint32_t h[256];
+template <typename K>
+__global__ void __launch_bounds__(RS_THREADS) radix_hist_kernel(const K *keys, int64_t n, int shift, int nd,
+                                                                uint32_t *counts, int ntiles) {
+    __shared__ uint32_t h[RS_DIGITS];
     h[threadIdx.x] = 0;
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * RS_TILE;
+#pragma unroll
     for (int i = 0; i < RS_ITEMS; ++i) {
         const int64_t k = base + (int64_t)i * RS_THREADS + threadIdx.x;
-        if (k < n) atomicAdd(&h[(keys[k] >> shift) & 0xFF], 1u);
+        if (k < n) atomicAdd(&h[(int)(keys[k] >> shift) & (nd - 1)], 1u);
     }
     __syncthreads();
-    counts[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+    if ((int)threadIdx.x < nd) counts[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
 }
 
-__global__ void radix_scatter_kernel(const uint64_t *keys, const uint32_t *vals, int64_t n, int shift,
-                                     const uint32_t *offsets, int ntiles, uint64_t *keys_out,
-                                     uint32_t *vals_out) {
-    __shared__ uint32_t wbase[RS_WARPS][256];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) (&wbase[0][0])[i] = 0;
+template <typename K>
+struct RadixSmem {
+    union {
+        K key[RS_TILE];
+        uint32_t val[RS_TILE];            // (after the keys have left)
+    };
+    uint32_t out[RS_DIGITS];              // output position of the digit's first key, less its place in the tile
+    uint16_t cnt[RS_WARPS][RS_DIGITS];    // running counts, then the digit's place before each warp
+    uint32_t wsum[RS_WARPS];
+};
+
+template <typename K>
+__global__ void __launch_bounds__(RS_THREADS, 2) radix_scatter_kernel(const K *keys, const uint32_t *vals, int64_t n,
+                                                                   int shift, int nd, const uint32_t *offsets,
+                                                                   int ntiles, K *keys_out, uint32_t *vals_out) {
+    extern __shared__ __align__(16) char rs_smem[];
+    RadixSmem<K> &sm = *reinterpret_cast<RadixSmem<K> *>(rs_smem);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int w = 0; w < RS_WARPS; ++w) sm.cnt[w][tid] = 0;
     __syncthreads();
-    const int64_t wstart = (int64_t)blockIdx.x * RS_TILE + (int64_t)warp * RS_ITEMS * 32;
-    uint64_t kk[RS_ITEMS];
+    const int64_t base = (int64_t)blockIdx.x * RS_TILE;
+    const int ntile = (int)min((int64_t)RS_TILE, n - base);
+    const int w0 = warp * RS_ITEMS * 32 + lane;        // the thread's first key of the tile
+    keys += base;
+    K kk[RS_ITEMS];
+    uint16_t rank[RS_ITEMS];
+#pragma unroll
+    for (int r = 0; r < RS_ITEMS; ++r) kk[r] = (w0 + r * 32 < ntile) ? keys[w0 + r * 32] : 0;
+    const unsigned lt = (1u << lane) - 1u;
+    // 1) rank among the warp's keys of the same digit
+    if (ntile == RS_TILE) {
+#pragma unroll
+        for (int r = 0; r < RS_ITEMS; ++r) {
+            const int d = (int)(kk[r] >> shift) & (nd - 1);
+            const unsigned peers = __match_any_sync(0xffffffffu, d);
+            const uint32_t before = sm.cnt[warp][d], mine = __popc(peers & lt);
+            rank[r] = (uint16_t)(before + mine);
+            __syncwarp();
+            if (mine == 0) sm.cnt[warp][d] = (uint16_t)(before + __popc(peers));
+            __syncwarp();
+        }
+    } else {
+        for (int r = 0; r < RS_ITEMS; ++r) {
+            const bool in = w0 + r * 32 < ntile;
+            const int d = in ? (int)(keys[w0 + r * 32] >> shift) & (nd - 1) : nd;   // (absent keys match one another)
+            const unsigned peers = __match_any_sync(0xffffffffu, d);
+            const uint32_t before = in ? sm.cnt[warp][d] : 0, mine = __popc(peers & lt);
+#pragma unroll
+            for (int q = 0; q < RS_ITEMS; ++q)
+                if (q == r) rank[q] = (uint16_t)(before + mine);
+            __syncwarp();
+            if (in && mine == 0) sm.cnt[warp][d] = (uint16_t)(before + __popc(peers));
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    // 2) a digit's place before each warp, its total, and the digits' places in the tile
+    uint32_t total = 0;
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) {
+        const uint32_t c = sm.cnt[w][tid];
+        sm.cnt[w][tid] = (uint16_t)total;
+        total += c;
+    }
+    uint32_t incl = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) sm.wsum[warp] = incl;
+    __syncthreads();
+    uint32_t place = incl - total;
+    for (int w = 0; w < warp; ++w) place += sm.wsum[w];
+    if (tid < nd) sm.out[tid] = offsets[(int64_t)tid * ntiles + blockIdx.x] - place;
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) sm.cnt[w][tid] += (uint16_t)place;
+    __syncthreads();
+    // 3) the keys in digit order, and out; then the values the same way (loaded while
+    // the keys leave)
+    uint16_t (&at)[RS_ITEMS] = rank;
+#pragma unroll
+    for (int r = 0; r < RS_ITEMS; ++r)
+        if (w0 + r * 32 < ntile) {
+            const int d = (int)(kk[r] >> shift) & (nd - 1);
+            at[r] = (uint16_t)(sm.cnt[warp][d] + rank[r]);
+            sm.key[at[r]] = kk[r];
+        }
     uint32_t vv[RS_ITEMS];
 #pragma unroll
-    for (int r = 0; r < RS_ITEMS; ++r) {
-        const int64_t k = wstart + r * 32 + lane;
-        kk[r] = (k < n) ? keys[k] : 0;
-        vv[r] = (k < n) ? vals[k] : 0;
-    }
-    const unsigned lt = (1u << lane) - 1u;
-    // 1) per-warp digit counts
+    for (int r = 0; r < RS_ITEMS; ++r)
+        vv[r] = w0 + r * 32 < ntile && vals ? __ldg(vals + base + w0 + r * 32) : (uint32_t)(base + w0 + r * 32);
+    __syncthreads();
+    uint32_t pos[RS_ITEMS];
 #pragma unroll
     for (int r = 0; r < RS_ITEMS; ++r) {
-        const int64_t k = wstart + r * 32 + lane;
-        const unsigned act = __ballot_sync(0xffffffffu, k < n);
-        if (k < n) {
-            const unsigned d = (unsigned)((kk[r] >> shift) & 0xFF);
-            const unsigned peers = __match_any_sync(act, d);
-            if ((peers & lt) == 0) wbase[warp][d] += __popc(peers);
-        }
-        __syncwarp();
-    }
-    __syncthreads();
-    // 2) warp bases: global tile offset + counts of the earlier warps
-    {
-        const int d = threadIdx.x;  // RS_THREADS == 256 digits
-        uint32_t run = offsets[(int64_t)d * ntiles + blockIdx.x];
-        for (int w = 0; w < RS_WARPS; ++w) {
-            const uint32_t c = wbase[w][d];
-            wbase[w][d] = run;
-            run += c;
+        const int i = r * RS_THREADS + tid;
+        if (i < ntile) {
+            const K key = sm.key[i];
+            pos[r] = sm.out[(int)(key >> shift) & (nd - 1)] + (uint32_t)i;
+            keys_out[pos[r]] = key;
         }
     }
     __syncthreads();
-    // 3) stable scatter, rounds in order
 #pragma unroll
     for (int r = 0; r < RS_ITEMS; ++r) {
-        const int64_t k = wstart + r * 32 + lane;
-        const unsigned act = __ballot_sync(0xffffffffu, k < n);
-        unsigned d = 0, peers = 0;
-        uint32_t pos = 0;
-        if (k < n) {
-            d = (unsigned)((kk[r] >> shift) & 0xFF);
-            peers = __match_any_sync(act, d);
-            pos = wbase[warp][d] + __popc(peers & lt);
-            keys_out[pos] = kk[r];
-            vals_out[pos] = vv[r];
-        }
-        __syncwarp();
-        if (k < n && (peers & lt) == 0) wbase[warp][d] += __popc(peers);
-        __syncwarp();
+        if (w0 + r * 32 < ntile) sm.val[at[r]] = vv[r];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RS_ITEMS; ++r) {
+        const int i = r * RS_THREADS + tid;
+        if (i < ntile) vals_out[pos[r]] = sm.val[i];
     }
 }
 
 // ------------------------------------------------------------ items
-__global__ void seg_flag_kernel(const uint64_t *keys, int64_t nvalid, int tb2, uint32_t *flag) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nvalid;
-         i += (int64_t)gridDim.x * blockDim.x)
-        flag[i] = (i == 0 || (keys[i] >> tb2) != (keys[i - 1] >> tb2)) ? 1u : 0u;
+// Starts of the segments of equal key >> shift, in two passes over the keys:
+// heads per block of SEG_BLOCK keys, and, after a scan of those counts, the heads
+// themselves.
+constexpr int SEG_THREADS = 256;
+constexpr int SEG_ITEMS = 8;
+constexpr int SEG_BLOCK = SEG_THREADS * SEG_ITEMS;
+
+template <typename K>
+__device__ __forceinline__ bool seg_head(const K *keys, int64_t i, int64_t n, int shift) {
+    return i < n && (i == 0 || (keys[i] >> shift) != (keys[i - 1] >> shift));
 }
 
-__global__ void seg_start_kernel(const uint32_t *flag, const uint32_t *segid, int64_t nvalid,
-                                 uint32_t *starts) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nvalid;
-         i += (int64_t)gridDim.x * blockDim.x)
-        if (flag[i]) starts[segid[i]] = (uint32_t)i;
+template <typename K>
+__global__ void __launch_bounds__(SEG_THREADS) seg_count_kernel(const K *keys, int64_t n, int shift, uint32_t *nhead) {
+    __shared__ uint32_t total;
+    if (threadIdx.x == 0) total = 0;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * SEG_BLOCK;
+    uint32_t c = 0;
+#pragma unroll
+    for (int r = 0; r < SEG_ITEMS; ++r)
+        c += __popc(__ballot_sync(0xffffffffu, seg_head(keys, base + r * SEG_THREADS + threadIdx.x, n, shift)));
+    if ((threadIdx.x & 31) == 0) atomicAdd(&total, c);
+    __syncthreads();
+    if (threadIdx.x == 0) nhead[blockIdx.x] = total;
+}
+
+template <typename K>
+__global__ void __launch_bounds__(SEG_THREADS) seg_start_kernel(const K *keys, int64_t n, int shift,
+                                                                const uint32_t *first, uint32_t *starts) {
+    __shared__ uint32_t wsum[SEG_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t at = first[blockIdx.x];
+    for (int r = 0; r < SEG_ITEMS; ++r) {
+        const int64_t i = (int64_t)blockIdx.x * SEG_BLOCK + r * SEG_THREADS + threadIdx.x;
+        const bool head = seg_head(keys, i, n, shift);
+        const unsigned m = __ballot_sync(0xffffffffu, head);
+        if (lane == 0) wsum[warp] = __popc(m);
+        __syncthreads();
+        uint32_t before = 0, all = 0;
+        for (int w = 0; w < SEG_THREADS / 32; ++w) {
+            if (w < warp) before += wsum[w];
+            all += wsum[w];
+        }
+        if (head) starts[at + before + __popc(m & ((1u << lane) - 1u))] = (uint32_t)i;
+        at += all;
+        __syncthreads();
+    }
 }
 
 __global__ void seg_chunks_kernel(const uint32_t *starts, int64_t nseg, uint32_t nvalid, int chunk,
@@ -301,28 +419,25 @@ __global__ void rg_emit_kernel(const uint32_t *starts, const uint32_t *base, int
     }
 }
 
-// REGION key of the i-th valid visibility (grid order): (bin, region tile
-// row, region tile column, oversampled offset) above the position inside the
-// tile (6 + 6 bits; tiles are at most 49 cells).  geo[bin].x = tile side (0: the
-// bin takes no region); those bins get invalid_key (sorted last); eligible
-// ones are counted in *nreg.
-__global__ void rg_key_kernel(const aw_rec *rec, int64_t nv, const int4 *geo, int OS, int osb, int nt,
-                              uint64_t invalid_key, uint64_t *keys, uint32_t *vals, unsigned long long *nreg) {
+// REGION key of the i-th visibility in degridding order: (bin, region tile row,
+// region tile column); the order by oversampled offset inside a bin and
+// super-tile is there already, and the sort is stable.  geo[bin].x = tile side
+// (0: the bin takes no region); those bins get invalid_key (sorted last);
+// eligible ones are counted in *nreg.
+template <typename K>
+__global__ void rg_key_kernel(const aw_rec *rec, int64_t nv, const int4 *geo, int nt, K invalid_key, K *keys,
+                              unsigned long long *nreg) {
     unsigned long long cnt = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nv;
          i += (int64_t)gridDim.x * blockDim.x) {
         const aw_rec r = rec[i];
         const int T = geo[r.bin].x;
-        uint64_t key = invalid_key;
+        K key = invalid_key;
         if (T > 0) {
-            const int ty = (int)r.y0 / T, tx = (int)r.x0 / T;
-            const int ly = (int)r.y0 - ty * T, lx = (int)r.x0 - tx * T;
-            const uint64_t grp = ((((uint64_t)r.bin * nt + ty) * nt + tx) << osb) | (uint64_t)(r.fy * OS + r.fx);
-            key = (grp << 12) | ((uint64_t)ly << 6) | (uint64_t)lx;
+            key = ((K)r.bin * nt + (int)r.y0 / T) * nt + (int)r.x0 / T;
             cnt++;
         }
         keys[i] = key;
-        vals[i] = (uint32_t)i;
     }
     for (int o = 16; o; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
     if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(nreg, cnt);
@@ -341,17 +456,14 @@ __global__ void rec_orig_kernel(const aw_rec *rec, int64_t n, uint32_t *perm) {
 }
 
 // Degridding key of the i-th valid visibility (grid order): (bin, super-tile
-// row, super-tile column, fy, fx) above the position inside the super-tile.
-__global__ void dg_key_kernel(const aw_rec *rec, int64_t nv, int OS, int stbits, int nst, uint64_t *keys,
-                              uint32_t *vals) {
-    const int smask = (1 << stbits) - 1;
+// row, super-tile column, fy, fx); inside a group the grid order (tile, then
+// position) stays.
+template <typename K>
+__global__ void dg_key_kernel(const aw_rec *rec, int64_t nv, int OS, int stbits, int nst, K *keys) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nv;
          i += (int64_t)gridDim.x * blockDim.x) {
         const aw_rec r = rec[i];
-        const uint64_t grp = (((uint64_t)r.bin * nst + (r.y0 >> stbits)) * nst + (r.x0 >> stbits)) * OS * OS +
-                             (uint64_t)r.fy * OS + r.fx;
-        keys[i] = (grp << (2 * stbits)) | ((uint64_t)(r.y0 & smask) << stbits) | (uint64_t)(r.x0 & smask);
-        vals[i] = (uint32_t)i;
+        keys[i] = (((K)r.bin * nst + (r.y0 >> stbits)) * nst + (r.x0 >> stbits)) * (OS * OS) + (int)r.fy * OS + r.fx;
     }
 }
 
@@ -380,7 +492,7 @@ int fill_coord_args(const aw_vis_desc *vis, const aw_kernel_set *ks, int tile, C
     a.uvw = vis->uvw;
     a.row = vis->row_of_vis;
     a.chan = vis->chan_of_vis;
-    a.freq = vis->freq;
+    a.fl = plan->d_fl;
     a.pa_bin = vis->pa_bin;
     a.fbin = vis->fbin;
     a.flags = vis->flags;
@@ -404,43 +516,62 @@ int fill_coord_args(const aw_vis_desc *vis, const aw_kernel_set *ks, int tile, C
     return AW_OK;
 }
 
-// LSD radix sort of (key, value) pairs over `passes` 8-bit digits; on return
-// k0/v0 point at the sorted arrays.  `counts`/`offs` hold 256 * ceil(n / RS_TILE)
-// words, `scratch` serves the exclusive scan of that many words.
-int radix_sort_pairs(uint64_t *&k0, uint32_t *&v0, uint64_t *&k1, uint32_t *&v1, int64_t n, int passes,
-                     uint32_t *counts, uint32_t *offs, void *scratch, cudaStream_t s) {
-    const int ntiles = (int)((n + RS_TILE - 1) / RS_TILE);
-    const int64_t ncounts = (int64_t)256 * ntiles;
-    for (int pass = 0; pass < passes; ++pass) {
-        const int shift = pass * 8;
-        radix_hist_kernel<<<ntiles, RS_THREADS, 0, s>>>(k0, n, shift, counts, ntiles);
-        AW_CHECK_LAUNCH();
-        int rc = aw_exclusive_scan_u32(counts, offs, ncounts, scratch, s);
-        if (rc) return rc;
-        radix_scatter_kernel<<<ntiles, RS_THREADS, 0, s>>>(k0, v0, n, shift, offs, ntiles, k1, v1);
-        AW_CHECK_LAUNCH();
-        std::swap(k0, k1);
-        std::swap(v0, v1);
+// One device allocation handed out in pieces (buf: freed with the arena, for the
+// temporaries; else the plan frees it).
+struct Arena {
+    DevBuf buf;
+    void *base = nullptr;
+    size_t size = 0, used = 0;
+    static size_t round(size_t b) { return (b + 255) / 256 * 256; }
+    template <class T>
+    T *take(size_t count) {
+        T *p = reinterpret_cast<T *>(static_cast<char *>(base) + used);
+        used += round(count * sizeof(T));
+        return p;
     }
-    return AW_OK;
+};
+
+// Sort buffers: two (key, value) arrays for n visibilities (64-bit keys), the
+// tile counts and their scan, and per-segment words.
+struct SortBufs {
+    uint64_t *k0, *k1;
+    uint32_t *v0, *v1;
+    uint32_t *words[3];   // max(tile counts, n + 1) words each
+    void *scratch;
+};
+
+int key_bits(uint64_t maxkey) {   // bits that hold 0 .. maxkey
+    int b = 1;
+    while (b < 64 && (maxkey >> b)) ++b;
+    return b;
 }
 
-// Starts of the segments of equal key >> shift in nv sorted keys; allocates
-// *starts.  `flag`/`segid` hold nv + 1 words each.
-int build_segments(const uint64_t *keys, int64_t nv, int shift, uint32_t *flag, uint32_t *segid, void *scratch,
-                   DevBuf &starts, int64_t *nseg, cudaStream_t s) {
-    seg_flag_kernel<<<grid_blocks(nv, 256), 256, 0, s>>>(keys, nv, shift, flag);
-    AW_CHECK_LAUNCH();
-    int rc = aw_exclusive_scan_u32(flag, segid, nv, scratch, s);
-    if (rc) return rc;
-    uint32_t last_id = 0, last_flag = 0;
-    AW_CUDA_TRY(cudaMemcpyAsync(&last_id, segid + nv - 1, 4, cudaMemcpyDeviceToHost, s));
-    AW_CUDA_TRY(cudaMemcpyAsync(&last_flag, flag + nv - 1, 4, cudaMemcpyDeviceToHost, s));
-    AW_CUDA_TRY(cudaStreamSynchronize(s));
-    *nseg = (int64_t)last_id + last_flag;
-    AW_CUDA_TRY(aw_dev_malloc(&starts.p, sizeof(uint32_t) * *nseg));
-    seg_start_kernel<<<grid_blocks(nv, 256), 256, 0, s>>>(flag, segid, nv, (uint32_t *)starts.p);
-    AW_CHECK_LAUNCH();
+// LSD radix sort of n keys of `bits` bits, the values being 0 .. n-1 at the
+// start; on return kin / vout point at the sorted arrays.
+template <typename K>
+int radix_sort(K *&kin, uint32_t *&vout, int64_t n, int bits, SortBufs &b, cudaStream_t s) {
+    const int ntiles = (int)((n + RS_TILE - 1) / RS_TILE);
+    const int passes = (bits + RS_BITS - 1) / RS_BITS, db = (bits + passes - 1) / passes, nd = 1 << db;
+    AW_CUDA_TRY(cudaFuncSetAttribute(radix_scatter_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sizeof(RadixSmem<K>)));
+    K *k0 = kin, *k1 = reinterpret_cast<K *>(kin == reinterpret_cast<K *>(b.k0) ? b.k1 : b.k0);
+    const uint32_t *v0 = nullptr;
+    uint32_t *v1 = b.v0;
+    for (int pass = 0; pass < passes; ++pass) {
+        const int shift = pass * db;
+        radix_hist_kernel<K><<<ntiles, RS_THREADS, 0, s>>>(k0, n, shift, nd, b.words[0], ntiles);
+        AW_CHECK_LAUNCH();
+        int rc = aw_exclusive_scan_u32(b.words[0], b.words[1], (int64_t)nd * ntiles, b.scratch, s);
+        if (rc) return rc;
+        radix_scatter_kernel<K><<<ntiles, RS_THREADS, sizeof(RadixSmem<K>), s>>>(k0, v0, n, shift, nd, b.words[1], ntiles,
+                                                                                k1, v1);
+        AW_CHECK_LAUNCH();
+        std::swap(k0, k1);
+        v0 = v1;
+        v1 = v1 == b.v0 ? b.v1 : b.v0;
+    }
+    kin = k0;
+    vout = const_cast<uint32_t *>(v0);
     return AW_OK;
 }
 
@@ -456,41 +587,49 @@ int scan_counts(const uint32_t *cnt, uint32_t *base, int64_t n, void *scratch, i
     return AW_OK;
 }
 
-// Cut the sorted keys of the nv valid visibilities into segments of equal
-// key >> shift and the segments into items of at most `chunk` visibilities;
-// allocates *items.  `flag`/`segid` hold nv + 1 words each.
-int build_items(const uint64_t *keys, int64_t nv, int shift, int chunk, const aw_rec *rec, uint32_t *flag,
-                uint32_t *segid, void *scratch, int4 **items, int64_t *nitems, cudaStream_t s) {
-    DevBuf bstarts, bnch, bbase;
-    int64_t nseg = 0;
-    int rc = build_segments(keys, nv, shift, flag, segid, scratch, bstarts, &nseg, s);
-    if (rc) return rc;
-    AW_CUDA_TRY(aw_dev_malloc(&bnch.p, sizeof(uint32_t) * nseg));
-    AW_CUDA_TRY(aw_dev_malloc(&bbase.p, sizeof(uint32_t) * nseg));
-    seg_chunks_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>((uint32_t *)bstarts.p, nseg, (uint32_t)nv, chunk,
-                                                            (uint32_t *)bnch.p);
+// Starts (b.words[2]) of the *nseg segments of equal key >> shift in nv sorted keys.
+template <typename K>
+int build_segments(const K *keys, int64_t nv, int shift, SortBufs &b, int64_t *nseg, cudaStream_t s) {
+    const int64_t nblk = (nv + SEG_BLOCK - 1) / SEG_BLOCK;
+    seg_count_kernel<K><<<(unsigned)nblk, SEG_THREADS, 0, s>>>(keys, nv, shift, b.words[0]);
     AW_CHECK_LAUNCH();
-    rc = scan_counts((uint32_t *)bnch.p, (uint32_t *)bbase.p, nseg, scratch, nitems, s);
+    const int rc = scan_counts(b.words[0], b.words[1], nblk, b.scratch, nseg, s);
     if (rc) return rc;
-    AW_CUDA_TRY(aw_dev_malloc(items, sizeof(int4) * std::max<int64_t>(*nitems, 1)));
-    emit_items_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>((uint32_t *)bstarts.p, (uint32_t *)bbase.p, nseg,
-                                                            (uint32_t)nv, chunk, rec, *items);
+    seg_start_kernel<K><<<(unsigned)nblk, SEG_THREADS, 0, s>>>(keys, nv, shift, b.words[1], b.words[2]);
     AW_CHECK_LAUNCH();
-    // the temporaries are freed on return: finish the kernels that read them
-    AW_CUDA_TRY(cudaStreamSynchronize(s));
     return AW_OK;
 }
 
-// The region tasks of the segments `starts` of the nreg records `rec` under the
-// per-bin geometry geo; allocates *tasks.  `cnt` and `base` hold nseg words each.
-int build_region_tasks(const uint32_t *starts, int64_t nseg, int64_t nreg, const aw_rec *rec, const int4 *geo,
-                       uint32_t *cnt, uint32_t *base, void *scratch, int4 **tasks, int64_t *ntasks, cudaStream_t s) {
-    rg_count_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>(starts, nseg, (uint32_t)nreg, rec, geo, cnt);
+// Cut the sorted keys of the nv valid visibilities into segments of equal
+// key >> shift and the segments into items of at most `chunk` visibilities;
+// allocates *items.
+template <typename K>
+int build_items(const K *keys, int64_t nv, int shift, int chunk, const aw_rec *rec, SortBufs &b, int4 **items,
+                int64_t *nitems, cudaStream_t s) {
+    int64_t nseg = 0;
+    int rc = build_segments<K>(keys, nv, shift, b, &nseg, s);
+    if (rc) return rc;
+    seg_chunks_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>(b.words[2], nseg, (uint32_t)nv, chunk, b.words[0]);
     AW_CHECK_LAUNCH();
-    const int rc = scan_counts(cnt, base, nseg, scratch, ntasks, s);
+    rc = scan_counts(b.words[0], b.words[1], nseg, b.scratch, nitems, s);
+    if (rc) return rc;
+    AW_CUDA_TRY(aw_dev_malloc(items, sizeof(int4) * std::max<int64_t>(*nitems, 1)));
+    emit_items_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>(b.words[2], b.words[1], nseg, (uint32_t)nv, chunk, rec,
+                                                            *items);
+    AW_CHECK_LAUNCH();
+    return AW_OK;
+}
+
+// The region tasks of the nseg segments (b.words[2]) of the nreg records `rec`
+// under the per-bin geometry geo; allocates *tasks.
+int build_region_tasks(int64_t nseg, int64_t nreg, const aw_rec *rec, const int4 *geo, SortBufs &b, int4 **tasks,
+                       int64_t *ntasks, cudaStream_t s) {
+    rg_count_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>(b.words[2], nseg, (uint32_t)nreg, rec, geo, b.words[0]);
+    AW_CHECK_LAUNCH();
+    const int rc = scan_counts(b.words[0], b.words[1], nseg, b.scratch, ntasks, s);
     if (rc) return rc;
     AW_CUDA_TRY(aw_dev_malloc(tasks, sizeof(int4) * std::max<int64_t>(*ntasks, 1)));
-    rg_emit_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>(starts, base, nseg, (uint32_t)nreg, rec, geo, *tasks);
+    rg_emit_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>(b.words[2], b.words[1], nseg, (uint32_t)nreg, rec, geo, *tasks);
     AW_CHECK_LAUNCH();
     return AW_OK;
 }
@@ -532,19 +671,42 @@ static int build_hybrid_items(aw_plan *plan, cudaStream_t s) {
 // the region kernel, its tasks, and the OFFSETS items of the other bins with
 // the second stream.  The region kernel is the faster one at every support it
 // takes (aw_rg_eligible), so every plane goes there, split_planes or not.
-// k0/v0/k1/v1 and the scan buffers are the plan builder's (>= nv).
-static int build_region(aw_plan *plan, const aw_kernel_set *ks, int64_t nv, uint64_t *k0, uint32_t *v0,
-                        uint64_t *k1, uint32_t *v1, uint32_t *counts, uint32_t *offs, void *scratch,
-                        cudaStream_t s) {
+// The sort buffers are the plan builder's (>= nv).
+template <typename K>
+static int sort_region(aw_plan *plan, int64_t nv, const int4 *d_geo, int nb, int nt, uint64_t maxkey,
+                       unsigned long long *d_nreg, SortBufs &b, cudaStream_t s) {
+    K *keys = reinterpret_cast<K *>(b.k0);
+    uint32_t *perm = nullptr;
+    rg_key_kernel<K><<<grid_blocks(nv, 256), 256, 0, s>>>(plan->d_rec_dg, nv, d_geo, nt, (K)maxkey, keys, d_nreg);
+    AW_CHECK_LAUNCH();
+    int rc = radix_sort<K>(keys, perm, nv, key_bits(maxkey), b, s);
+    if (rc) return rc;
+    unsigned long long nreg = 0;
+    AW_CUDA_TRY(cudaMemcpyAsync(&nreg, d_nreg, sizeof(nreg), cudaMemcpyDeviceToHost, s));
+    AW_CUDA_TRY(cudaStreamSynchronize(s));
+    plan->nreg = (int64_t)nreg;
+    if (plan->nreg == 0) return AW_OK;
+    gather_rec_kernel<<<grid_blocks(plan->nreg, 256), 256, 0, s>>>(plan->d_rec_dg, perm, plan->nreg, plan->d_rec_rg);
+    AW_CHECK_LAUNCH();
+    int64_t nseg = 0;
+    rc = build_segments<K>(keys, plan->nreg, 0, b, &nseg, s);
+    if (rc == AW_OK)
+        rc = build_region_tasks(nseg, plan->nreg, plan->d_rec_rg, d_geo, b, &plan->d_items_rg, &plan->nitems_rg, s);
+    if (rc == AW_OK && plan->npol == 1)
+        rc = build_region_tasks(nseg, plan->nreg, plan->d_rec_rg, d_geo + nb, b, &plan->d_items_rgd, &plan->nitems_rgd, s);
+    return rc;
+}
+
+static int build_region(aw_plan *plan, const aw_kernel_set *ks, int64_t nv, SortBufs &b, cudaStream_t s) {
     const int nb = ks->nbins;
     // gridding geometry of every bin, then the degridding one
     std::vector<int4> geo((size_t)nb * 2, make_int4(0, 0, 0, 0));
     bool all = true;
-    for (int b = 0; b < nb; ++b) {
-        const int S = ks->bin_support[(size_t)b];
+    for (int i = 0; i < nb; ++i) {
+        const int S = ks->bin_support[(size_t)i];
         if (aw_rg_eligible(S, plan->npol)) {
-            geo[(size_t)b] = make_int4(aw_rg_tile(S), AW_RG_MAXV, aw_rg_nblk(S), 0);
-            geo[(size_t)nb + b] = make_int4(aw_rg_tile(S), AW_RG_MAXV_DG, 1, 0);
+            geo[(size_t)i] = make_int4(aw_rg_tile(S), AW_RG_MAXV, aw_rg_nblk(S), 0);
+            geo[(size_t)nb + i] = make_int4(aw_rg_tile(S), AW_RG_MAXV_DG, 1, 0);
         } else {
             all = false;
         }
@@ -552,51 +714,15 @@ static int build_region(aw_plan *plan, const aw_kernel_set *ks, int64_t nv, uint
     DevBuf dgeo, dcnt;
     AW_CUDA_TRY(aw_dev_malloc(&dgeo.p, sizeof(int4) * geo.size()));
     AW_CUDA_TRY(cudaMemcpyAsync(dgeo.p, geo.data(), sizeof(int4) * geo.size(), cudaMemcpyHostToDevice, s));
-    const int4 *d_geo = (const int4 *)dgeo.p;
     AW_CUDA_TRY(aw_dev_malloc(&dcnt.p, sizeof(unsigned long long)));
     AW_CUDA_TRY(cudaMemsetAsync(dcnt.p, 0, sizeof(unsigned long long), s));
-    AW_CUDA_TRY(aw_dev_malloc(&plan->d_rcounter, sizeof(unsigned int) * AW_RG_COUNTERS));
-    const int OS = plan->OS;
-    const int osb = ilog2(OS * OS);
     const int nt = (plan->N + aw_rg_tile(128) - 1) / aw_rg_tile(128);   // tiles an axis at the smallest tile side
-    const uint64_t maxgrp = ((uint64_t)nb * nt * nt) << osb;
-    int gbits = 0;
-    while (gbits < 63 && (1ull << gbits) <= maxgrp) ++gbits;
-    if (gbits + 12 > 62) return aw_set_error(AW_EINVAL, "region key needs %d bits", gbits + 12);
-    const int kbits = gbits + 12;
-    const uint64_t invalid_key = 1ull << kbits;
-    rg_key_kernel<<<grid_blocks(nv, 256), 256, 0, s>>>(plan->d_rec, nv, d_geo, OS, osb, nt, invalid_key, k0, v0,
-                                                      (unsigned long long *)dcnt.p);
-    AW_CHECK_LAUNCH();
-    int rc = radix_sort_pairs(k0, v0, k1, v1, nv, (kbits + 1 + 7) / 8, counts, offs, scratch, s);
+    const uint64_t maxkey = (uint64_t)nb * nt * nt;                     // also the key of the bins that take no region
+    const int4 *d_geo = (const int4 *)dgeo.p;
+    unsigned long long *d_nreg = (unsigned long long *)dcnt.p;
+    const int rc = key_bits(maxkey) <= 32 ? sort_region<uint32_t>(plan, nv, d_geo, nb, nt, maxkey, d_nreg, b, s)
+                                          : sort_region<uint64_t>(plan, nv, d_geo, nb, nt, maxkey, d_nreg, b, s);
     if (rc) return rc;
-    unsigned long long nreg = 0;
-    AW_CUDA_TRY(cudaMemcpyAsync(&nreg, dcnt.p, sizeof(nreg), cudaMemcpyDeviceToHost, s));
-    AW_CUDA_TRY(cudaStreamSynchronize(s));
-    plan->nreg = (int64_t)nreg;
-    AW_CUDA_TRY(aw_dev_malloc(&plan->d_rec_rg, sizeof(aw_rec) * std::max<int64_t>(plan->nreg, 1)));
-    if (plan->nreg > 0) {
-        gather_rec_kernel<<<grid_blocks(plan->nreg, 256), 256, 0, s>>>(plan->d_rec, v0, plan->nreg, plan->d_rec_rg);
-        AW_CHECK_LAUNCH();
-        DevBuf bstarts, bcnt, bbase;
-        int64_t nseg = 0;
-        rc = build_segments(k0, plan->nreg, osb + 12, counts, offs, scratch, bstarts, &nseg, s);
-        if (rc) return rc;
-        AW_CUDA_TRY(aw_dev_malloc(&bcnt.p, sizeof(uint32_t) * nseg));
-        AW_CUDA_TRY(aw_dev_malloc(&bbase.p, sizeof(uint32_t) * nseg));
-        const uint32_t *starts = (const uint32_t *)bstarts.p;
-        uint32_t *cnt = (uint32_t *)bcnt.p, *base = (uint32_t *)bbase.p;
-        rc = build_region_tasks(starts, nseg, plan->nreg, plan->d_rec_rg, d_geo, cnt, base, scratch,
-                                &plan->d_items_rg, &plan->nitems_rg, s);
-        if (rc) return rc;
-        if (plan->npol == 1) {
-            rc = build_region_tasks(starts, nseg, plan->nreg, plan->d_rec_rg, d_geo + nb, cnt, base, scratch,
-                                    &plan->d_items_rgd, &plan->nitems_rgd, s);
-            if (rc) return rc;
-        }
-        // the temporaries are freed here: finish the kernels that read them
-        AW_CUDA_TRY(cudaStreamSynchronize(s));
-    }
     // the other bins: their degridding items on the OFFSETS schedule
     if (!all) {
         std::vector<int4> hd((size_t)plan->nitems_dg), keep;
@@ -671,96 +797,116 @@ int aw_plan_build(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *ks, 
     // per-plane supports first (the coordinate step indexes by w plane), then per bin
     std::vector<int32_t> sup(ks->supports.begin(), ks->supports.end());
     plan->bin_support = ks->bin_support;
+    const int64_t n = vis->nvis;
+    const int nchan = std::max(vis->nchan, 1);
+    const bool region = t.grid_mode == AW_GRID_REGION;
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_plane_support, sizeof(int32_t) * std::max<size_t>(sup.size(), 1)));
-    AW_CUDA_TRY(cudaMemcpy(plan->d_plane_support, sup.data(), sizeof(int32_t) * sup.size(), cudaMemcpyHostToDevice));
+    AW_CUDA_TRY(aw_dev_malloc(&plan->d_fl, sizeof(double) * nchan));
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_wsum, sizeof(double)));
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_nonfinite, sizeof(unsigned long long)));
-    AW_CUDA_TRY(aw_dev_malloc(&plan->d_counter, sizeof(unsigned int) * 4));
-    const int64_t n = vis->nvis;
-    AW_CUDA_TRY(aw_dev_malloc(&plan->d_rec, sizeof(aw_rec) * std::max<int64_t>(n, 1)));
+    AW_CUDA_TRY(aw_dev_malloc(&plan->d_counter, sizeof(unsigned int) * (4 + AW_RG_COUNTERS)));
+    plan->d_rcounter = plan->d_counter + 4;
+    // the records of the plan's orders, in one allocation
+    Arena keep;
+    keep.size = (region ? 3 : 2) * Arena::round(sizeof(aw_rec) * std::max<int64_t>(n, 1));
+    AW_CUDA_TRY(aw_dev_malloc(&plan->d_block, keep.size));
+    keep.base = plan->d_block;
+    plan->d_rec = keep.take<aw_rec>(n);
+    plan->d_rec_dg = keep.take<aw_rec>(n);
+    if (region) plan->d_rec_rg = keep.take<aw_rec>(n);
+    AW_CUDA_TRY(cudaMemcpyAsync(plan->d_plane_support, sup.data(), sizeof(int32_t) * sup.size(),
+                                cudaMemcpyHostToDevice, s));
     if (n == 0) {
         AW_CUDA_TRY(aw_dev_malloc(&plan->d_items, sizeof(int4)));
+        AW_CUDA_TRY(cudaStreamSynchronize(s));
         return AW_OK;
+    }
+    if (vis->nchan > 0) {
+        channel_kernel<<<grid_blocks(vis->nchan, 256), 256, 0, s>>>(vis->freq, vis->nchan, plan->d_fl);
+        AW_CHECK_LAUNCH();
     }
     CoordArgs a;
     fill_coord_args(vis, ks, t.tile, a, plan);
     plan->uscale = a.uscale;
     plan->half = a.half;
     plan->winv = a.winv;
-    // key width: bins x tiles x (tile position), plus one bit for invalid
+    // keys: bins x tiles x (tile position), and one value for invalid ones
     const uint64_t maxkey = ((uint64_t)ks->nbins * a.nty * a.ntx) << (2 * a.tbits);
-    int kbits = 0;
-    while (kbits < 63 && (1ull << kbits) <= maxkey) ++kbits;
-    const uint64_t invalid_key = 1ull << kbits;
-    const int passes = (kbits + 1 + 7) / 8;
+    const int kbits = key_bits(maxkey);
 
-    DevBuf bk0, bk1, bv0, bv1, brec, bcnt, bcounts, bscan, bscratch;
-    AW_CUDA_TRY(aw_dev_malloc(&bk0.p, sizeof(uint64_t) * n));
-    AW_CUDA_TRY(aw_dev_malloc(&bk1.p, sizeof(uint64_t) * n));
-    AW_CUDA_TRY(aw_dev_malloc(&bv0.p, sizeof(uint32_t) * n));
-    AW_CUDA_TRY(aw_dev_malloc(&bv1.p, sizeof(uint32_t) * n));
-    AW_CUDA_TRY(aw_dev_malloc(&brec.p, sizeof(aw_rec) * n));
-    AW_CUDA_TRY(aw_dev_malloc(&bcnt.p, sizeof(unsigned long long) * 4));
-    AW_CUDA_TRY(cudaMemsetAsync(bcnt.p, 0, sizeof(unsigned long long) * 4, s));
-    uint64_t *k0 = (uint64_t *)bk0.p, *k1 = (uint64_t *)bk1.p;
-    uint32_t *v0 = (uint32_t *)bv0.p, *v1 = (uint32_t *)bv1.p;
-    coords_kernel<<<grid_blocks(n, 256), 256, 0, s>>>(a, invalid_key, k0, v0, (aw_rec *)brec.p,
-                                                     (unsigned long long *)bcnt.p);
-    AW_CHECK_LAUNCH();
-    // radix sort passes
-    const int ntiles = (int)((n + RS_TILE - 1) / RS_TILE);
-    const int64_t ncounts = (int64_t)256 * ntiles;
-    const int64_t scan_n = std::max<int64_t>(ncounts, n + 1);
-    AW_CUDA_TRY(aw_dev_malloc(&bcounts.p, sizeof(uint32_t) * scan_n));
-    AW_CUDA_TRY(aw_dev_malloc(&bscan.p, sizeof(uint32_t) * scan_n));
-    AW_CUDA_TRY(aw_dev_malloc(&bscratch.p, aw_scan_scratch_bytes(scan_n)));
-    uint32_t *counts = (uint32_t *)bcounts.p, *offs = (uint32_t *)bscan.p;
-    int rc = radix_sort_pairs(k0, v0, k1, v1, n, passes, counts, offs, bscratch.p, s);
-    if (rc) return rc;
-    gather_rec_kernel<<<grid_blocks(n, 256), 256, 0, s>>>((aw_rec *)brec.p, v0, n, plan->d_rec);
-    AW_CHECK_LAUNCH();
-    unsigned long long hc[4];
-    AW_CUDA_TRY(cudaMemcpyAsync(hc, bcnt.p, sizeof(hc), cudaMemcpyDeviceToHost, s));
-    AW_CUDA_TRY(cudaStreamSynchronize(s));
-    plan->n_outside = (int64_t)hc[0];
-    plan->n_flagged = (int64_t)hc[1];
-    plan->nvalid = (int64_t)hc[2];
-    plan->mean_taps = hc[2] ? (double)hc[3] / (double)hc[2] : 0.0;
+    // the temporaries, in one allocation
+    const int64_t ntiles = (n + RS_TILE - 1) / RS_TILE;
+    const size_t words = (size_t)std::max<int64_t>(ntiles * RS_DIGITS, n + 1);
+    Arena ar;
+    ar.size = 2 * Arena::round(sizeof(uint64_t) * n) + 2 * Arena::round(sizeof(uint32_t) * n) +
+              Arena::round(sizeof(aw_rec) * n) + 3 * Arena::round(sizeof(uint32_t) * words) +
+              Arena::round(aw_scan_scratch_bytes((int64_t)words)) + Arena::round(sizeof(unsigned long long) * 4);
+    AW_CUDA_TRY(aw_dev_malloc(&ar.buf.p, ar.size));
+    ar.base = ar.buf.p;
+    SortBufs b;
+    b.k0 = ar.take<uint64_t>(n);
+    b.k1 = ar.take<uint64_t>(n);
+    b.v0 = ar.take<uint32_t>(n);
+    b.v1 = ar.take<uint32_t>(n);
+    aw_rec *rec = ar.take<aw_rec>(n);
+    for (auto &w : b.words) w = ar.take<uint32_t>(words);
+    b.scratch = ar.take<char>(aw_scan_scratch_bytes((int64_t)words));
+    unsigned long long *d_cnt = ar.take<unsigned long long>(4);
+    AW_CUDA_TRY(cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long) * 4, s));
+    // the gridding order and its items: runs of equal (bin, tile), then chunks
+    auto grid_order = [&](auto key) -> int {
+        using K = decltype(key);
+        K *keys = reinterpret_cast<K *>(b.k0);
+        uint32_t *perm = nullptr;
+        coords_kernel<K><<<grid_blocks(n, 256), 256, 0, s>>>(a, (K)maxkey, keys, rec, d_cnt);
+        AW_CHECK_LAUNCH();
+        int rc = radix_sort<K>(keys, perm, n, kbits, b, s);
+        if (rc) return rc;
+        gather_rec_kernel<<<grid_blocks(n, 256), 256, 0, s>>>(rec, perm, n, plan->d_rec);
+        AW_CHECK_LAUNCH();
+        unsigned long long hc[4];
+        AW_CUDA_TRY(cudaMemcpyAsync(hc, d_cnt, sizeof(hc), cudaMemcpyDeviceToHost, s));
+        AW_CUDA_TRY(cudaStreamSynchronize(s));
+        plan->n_outside = (int64_t)hc[0];
+        plan->n_flagged = (int64_t)hc[1];
+        plan->nvalid = (int64_t)hc[2];
+        plan->mean_taps = hc[2] ? (double)hc[3] / (double)hc[2] : 0.0;
+        if (plan->nvalid == 0) {
+            AW_CUDA_TRY(aw_dev_malloc(&plan->d_items, sizeof(int4)));
+            plan->nitems = 0;
+            return AW_OK;
+        }
+        return build_items<K>(keys, plan->nvalid, 2 * a.tbits, t.chunk, plan->d_rec, b, &plan->d_items,
+                              &plan->nitems, s);
+    };
+    int rc = kbits <= 32 ? grid_order(uint32_t()) : grid_order(uint64_t());
+    if (rc || plan->nvalid == 0) return rc;
     const int64_t nv = plan->nvalid;
-    if (nv == 0) {
-        AW_CUDA_TRY(aw_dev_malloc(&plan->d_items, sizeof(int4)));
-        plan->nitems = 0;
-        return AW_OK;
-    }
-    // gridding items: runs of equal (bin, tile), then chunks
-    rc = build_items(k0, nv, 2 * a.tbits, t.chunk, plan->d_rec, counts, offs, bscratch.p, &plan->d_items,
-                     &plan->nitems, s);
-    if (rc) return rc;
 
-    // degridding order: (bin, super-tile, oversampled offset, position in super-tile)
+    // degridding order: (bin, super-tile, oversampled offset), the grid order inside
     const int stbits = ilog2(plan->dg_tile);
     const int nst = (sp.N + plan->dg_tile - 1) >> stbits;
     const uint64_t ngroups = (uint64_t)ks->nbins * nst * nst * sp.OS * sp.OS;
-    const uint64_t dg_maxkey = ngroups << (2 * stbits);
-    int dg_bits = 0;
-    while (dg_bits < 63 && (1ull << dg_bits) <= dg_maxkey) ++dg_bits;
-    if (dg_bits > 62) return aw_set_error(AW_EINVAL, "degridding key needs %d bits; raise dg_tile", dg_bits);
-    dg_key_kernel<<<grid_blocks(nv, 256), 256, 0, s>>>(plan->d_rec, nv, sp.OS, stbits, nst, k0, v0);
-    AW_CHECK_LAUNCH();
-    rc = radix_sort_pairs(k0, v0, k1, v1, nv, (dg_bits + 7) / 8, counts, offs, bscratch.p, s);
-    if (rc) return rc;
-    AW_CUDA_TRY(aw_dev_malloc(&plan->d_rec_dg, sizeof(aw_rec) * nv));
-    gather_rec_kernel<<<grid_blocks(nv, 256), 256, 0, s>>>(plan->d_rec, v0, nv, plan->d_rec_dg);
-    AW_CHECK_LAUNCH();
-    rc = build_items(k0, nv, 2 * stbits, AW_DG_CHUNK, plan->d_rec_dg, counts, offs, bscratch.p,
-                     &plan->d_items_dg, &plan->nitems_dg, s);
+    auto degrid_order = [&](auto key) -> int {
+        using K = decltype(key);
+        K *keys = reinterpret_cast<K *>(b.k0);
+        uint32_t *perm = nullptr;
+        dg_key_kernel<K><<<grid_blocks(nv, 256), 256, 0, s>>>(plan->d_rec, nv, sp.OS, stbits, nst, keys);
+        AW_CHECK_LAUNCH();
+        int r = radix_sort<K>(keys, perm, nv, key_bits(ngroups), b, s);
+        if (r) return r;
+        gather_rec_kernel<<<grid_blocks(nv, 256), 256, 0, s>>>(plan->d_rec, perm, nv, plan->d_rec_dg);
+        AW_CHECK_LAUNCH();
+        return build_items<K>(keys, nv, 0, AW_DG_CHUNK, plan->d_rec_dg, b, &plan->d_items_dg, &plan->nitems_dg, s);
+    };
+    rc = key_bits(ngroups) <= 32 ? degrid_order(uint32_t()) : degrid_order(uint64_t());
     if (rc) return rc;
     if (t.grid_mode == AW_GRID_HYBRID) {
         rc = build_hybrid_items(plan, s);
         if (rc) return rc;
     }
     if (t.grid_mode == AW_GRID_REGION) {
-        rc = build_region(plan, ks, nv, k0, v0, k1, v1, counts, offs, bscratch.p, s);
+        rc = build_region(plan, ks, nv, b, s);
         if (rc) return rc;
     }
     AW_CUDA_TRY(cudaStreamSynchronize(s));
@@ -778,7 +924,7 @@ int aw_plan_coords_impl(const aw_plan *plan, const aw_kernel_set *ks_unused, int
     a.uvw = vis->uvw;
     a.row = vis->row_of_vis;
     a.chan = vis->chan_of_vis;
-    a.freq = vis->freq;
+    a.fl = plan->d_fl;
     a.pa_bin = vis->pa_bin;
     a.fbin = vis->fbin;
     a.flags = vis->flags;

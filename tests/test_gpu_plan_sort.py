@@ -1,0 +1,48 @@
+"""GPU: the plan's sorts at the edges of their tiles (8192 keys) and key widths
+(32 and 64 bits): the grid order is numpy's stable sort of the same keys, far-out
+and non-finite coordinates come last, and the degridding items are the groups'."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("wide", [False, True])
+@pytest.mark.parametrize("n", [1, 31, 8191, 8192, 8193, 40001])
+def test_orders(n, wide):
+    from paper_2206_15117_gb300 import aw
+    ctx = aw.aw_create(0)
+    # (bin, tile, position) needs 33 bits when wide, 20 otherwise
+    N, nw, npa, nfb = (4096, 8, 8, 8) if wide else (256, 2, 3, 2)
+    rng = np.random.default_rng(n + wide)
+    uvw = rng.uniform(-1.0, 1.0, (500, 3)) * 55.0
+    uvw[7], uvw[8], uvw[9] = (np.inf, 0.0, 1.0), (1.0, np.nan, np.nan), (1e300, 1.0, -np.inf)
+    row, chan = rng.integers(0, 500, n).astype(np.int32), rng.integers(0, 5, n).astype(np.int16)
+    pa, fb = rng.integers(0, npa, 500).astype(np.uint8), rng.integers(0, nfb, 5).astype(np.uint8)
+    freq = np.linspace(1.2e9, 1.5e9, 5)
+    kw = dict(N=N, dl=0.4 / 256, OS=4, npol=4, nw=nw, w_max=270.0, supports=[8] * nw, pa=[0.1 * i for i in range(npa)],
+              fbin_freqs=[1.3e9] * nfb)
+    if wide:
+        kw["dl"] = 1.0 / 4096
+    ks = aw.aw_make_kernels(ctx, **kw)
+    dev = [torch.as_tensor(x, device="cuda") for x in (uvw, row, chan, freq, pa, fb)]
+    plan = aw.aw_plan_create(ctx, aw.vis_desc(*dev), ks, aw.aw_tune(32, 256, 2, 256, aw.AW_GRID_REGION))
+    out = {k: torch.empty(n, dtype=torch.int32, device="cuda") for k in ("x0", "y0", "fx", "fy", "bin")}
+    valid, flip = (torch.empty(n, dtype=torch.uint8, device="cuda") for _ in range(2))
+    perm = torch.empty(n, dtype=torch.int32, device="cuda")
+    aw.aw_plan_coords(plan, **out, flip=flip, valid=valid)
+    aw.aw_plan_order(plan, perm)
+    c = {k: v.cpu().numpy().astype(np.int64) for k, v in out.items()}
+    ok = valid.cpu().numpy() == 1
+    bad = np.isin(row, (7, 8, 9))
+    assert not ok[bad].any() and np.all(c["x0"][bad] == 0)
+    np.testing.assert_array_equal(flip.cpu().numpy() == 1, (uvw[row, 2] < 0))
+    nt = N // 32
+    key = ((c["bin"] * nt + c["y0"] // 32) * nt + c["x0"] // 32) * 1024 + c["y0"] % 32 * 32 + c["x0"] % 32
+    key[~ok] = 1 << 60
+    np.testing.assert_array_equal(perm.cpu().numpy(), np.argsort(key, kind="stable"))
+    grp = ((c["bin"] * 64 + c["y0"] // 256) * 64 + c["x0"] // 256) * 16 + c["fy"] * 4 + c["fx"]
+    cnt = np.unique(grp[ok], return_counts=True)[1]
+    info = aw.aw_plan_query(plan)
+    assert info.nitems_degrid == int(((cnt + 31) // 32).sum()) and info.nvalid == int(ok.sum())
