@@ -110,86 +110,77 @@ __device__ __noinline__ void reproject_pixel64(const ReprojArgs &a, int qx, int 
     sample<INTERP>(a, i, (int)fx + O, (int)fy + O, (float)(x - fx), (float)(y - fy));
 }
 
-// Source position of a tile's pixels as a Taylor expansion about the tile
-// centre, in fixed point with RP_FRAC fraction bits: X + a Ax + b Bx plus a
-// polynomial of degrees 2 and 3 in the pixel offsets (a, b), which only the
-// direction cosine n = sqrt(1 - l^2 - m^2) contributes.
+// Source position of a tile's pixels (a, b) columns and rows from its centre, in
+// fixed point with RP_FRAC fraction bits: X + a A + b B is exact in the direction
+// cosines l, m and linear in n = sqrt(1 - l^2 - m^2); the rest of n is added in FP32.
 constexpr int RP_FRAC = 40;
 constexpr int RP_TX = 64, RP_TY = 32;
 struct TilePos {
-    long long X, Ax, Bx, Y, Ay, By;
-    float q[7];          // n's coefficients of a^2, ab, b^2, a^3, a^2 b, a b^2, b^3
-    float qx, qy;        // R[2], R[5] over the source pixel size
-    int state;           // 0: every pixel in FP64, 1: expansion, 2: nothing but fill
+    long long X[2], A[2], B[2];   // x and y: at the centre, per column, per row
+    float rs[2];                  // R[2], R[5] over the source pixel size
+    float l, m, n;                // direction cosines of the centre
+    int ok[3], out[2];
 };
 
 // A CTA takes a tile of 64 x 32 destination pixels.  FP64 is slow on this part:
-// one thread expands the position map about the tile centre in FP64, the others
-// evaluate it in 64-bit integers.  The expansion is used where its remainder is
-// below 2^-25 pixels, under the FP32 rounding of the interpolation weights (else
-// the tile's pixels take the FP64 form).  Where a position lies so close to a
-// whole pixel that its rounding could decide whether the stencil is inside the
-// image, the pixel is done in FP64.  Seven fields of 2048^2 x 4 onto 4096^2 x 4
-// with their weights and combination: 5.40 -> 2.15 ms (2.00 with the beams of
-// mosaic_gamma read once); about a third of it now is the mosaic frame's writes.
+// the position map is expanded about the tile centre in FP64 once and evaluated
+// for the pixels in 64-bit integers.  What n departs from its linear part by comes
+// from the difference of squares, with no cancellation, so FP32 gives it to a few
+// 1e-7 of itself; it has to be below 0.05 pixels (else the tile's pixels take the
+// FP64 form), which leaves the position within the FP32 rounding of the
+// interpolation weights.  Where a position lies so close to a whole pixel that its
+// rounding could decide whether the stencil is inside the image, the pixel is done
+// in FP64.  Seven fields of 2048^2 x 4 onto 4096^2 x 4 with their weights and
+// combination: 5.37 -> 1.66 ms; one field 620 -> 158 us, of 256^2 onto 400^2
+// 17.1 -> 16.7 us.
 template <int INTERP>
 __global__ void __launch_bounds__(256) reproject_kernel(ReprojArgs a) {
     constexpr int K = (INTERP == AW_INTERP_CUBIC) ? 4 : 2;
     constexpr int O = (INTERP == AW_INTERP_CUBIC) ? -1 : 0;
     __shared__ TilePos tp;
     const int x0t = blockIdx.x * RP_TX, y0t = blockIdx.y * RP_TY;
-    if (threadIdx.x == 0) {
-        TilePos t{};
+    // the lead lanes of three warps share the FP64 work: a small image waits for its latency
+    const int role = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0 && role < 3) {
         const double l = ((double)(x0t + RP_TX / 2) - a.cx_d) * a.dl_d;
         const double m = ((double)(y0t + RP_TY / 2) - a.cy_d) * a.dl_d;
         const double n2 = 1.0 - l * l - m * m;
-        const double dmax = a.dl_d * 36.0;   // farthest offset in the tile: sqrt(32^2 + 16^2) = 35.8
-        t.state = 0;
-        if (n2 > 0.1 && dmax < 0.02) {
-            const double i1 = rsqrt(n2), n = n2 * i1, i2 = i1 * i1, i3 = i2 * i1, i5 = i3 * i2;
-            const double nl = -l * i1, nm = -m * i1;
-            const double d = a.dl_d, s = a.inv_dl_s;
-            const double x = (a.R[0] * l + a.R[1] * m + a.R[2] * n) * s + a.cx_s;
-            const double y = (a.R[3] * l + a.R[4] * m + a.R[5] * n) * s + a.cy_s;
+        const double i1 = rsqrt(fmax(n2, 0.05)), n = n2 * i1;   // (used for n^2 > 0.05 only)
+        const double s = a.inv_dl_s;
+        if (role < 2) {
+            // x or y at the centre and its slopes
+            const double r0 = a.R[3 * role], r1 = a.R[3 * role + 1], r2 = a.R[3 * role + 2];
+            const double ds = a.dl_d * s;
+            const double x = (r0 * l + r1 * m + r2 * n) * s + (role ? a.cy_s : a.cx_s);
+            const double ax = (r0 - r2 * (l * i1)) * ds, bx = (r1 - r2 * (m * i1)) * ds;
+            const double reach = 64.0 * fmax(fabs(ax), fabs(bx)) + 4.0;
+            const bool ok = reach < 4096.0 && fabs(x) < 4.0e6;
+            const double one = (double)(1ll << RP_FRAC);
+            tp.X[role] = ok ? llrint(x * one) : 0;
+            tp.A[role] = ok ? llrint(ax * one) : 0;
+            tp.B[role] = ok ? llrint(bx * one) : 0;
+            tp.rs[role] = (float)(r2 * s);
+            tp.ok[role] = ok;
+            // every stencil of the tile well outside the image
+            tp.out[role] = x < (double)(-O) - 1.0 - reach || x > (double)(a.Ns - K - O) + 1.0 + reach;
+        } else {
+            const double dmax = a.dl_d * 36.0;   // farthest offset in the tile: sqrt(32^2 + 16^2) = 35.8
+            const double rest = 2.0 * dmax * dmax * (i1 * i1) * i1 * s * fmax(fabs(a.R[2]), fabs(a.R[5]));
             const double z = a.R[6] * l + a.R[7] * m + a.R[8] * n;
-            const double ax = (a.R[0] + a.R[2] * nl) * d * s, bx = (a.R[1] + a.R[2] * nm) * d * s;
-            const double ay = (a.R[3] + a.R[5] * nl) * d * s, by = (a.R[4] + a.R[5] * nm) * d * s;
-            // remainder: the fourth derivative of n along a line is at most 15 / n^7, n^2 > 0.06 in
-            // the tile, so dmax^4 / 24 of it is below 4 dmax^4 / n^7 at the centre
-            const double rem = dmax * dmax * dmax * dmax * i5 * i2 * 4.0 * s * fmax(fabs(a.R[2]), fabs(a.R[5]));
-            const double reach = 64.0 * fmax(fmax(fabs(ax), fabs(bx)), fmax(fabs(ay), fabs(by))) + 4.0;
-            if (rem < 2.9e-8 && z > 0.1 && reach < 4096.0 && fabs(x) < 4.0e6 && fabs(y) < 4.0e6) {
-                const double one = (double)(1ll << RP_FRAC);
-                t.state = 1;
-                t.X = llrint(x * one);
-                t.Y = llrint(y * one);
-                t.Ax = llrint(ax * one);
-                t.Bx = llrint(bx * one);
-                t.Ay = llrint(ay * one);
-                t.By = llrint(by * one);
-                const double d2 = d * d, d3 = d2 * d;
-                t.q[0] = (float)(-0.5 * (1.0 - m * m) * i3 * d2);
-                t.q[1] = (float)(-l * m * i3 * d2);
-                t.q[2] = (float)(-0.5 * (1.0 - l * l) * i3 * d2);
-                t.q[3] = (float)(-0.5 * l * (1.0 - m * m) * i5 * d3);
-                t.q[4] = (float)(-0.5 * m * (1.0 + 2.0 * l * l - m * m) * i5 * d3);
-                t.q[5] = (float)(-0.5 * l * (1.0 + 2.0 * m * m - l * l) * i5 * d3);
-                t.q[6] = (float)(-0.5 * m * (1.0 - l * l) * i5 * d3);
-                t.qx = (float)(a.R[2] * s);
-                t.qy = (float)(a.R[5] * s);
-                // every stencil of the tile well outside the image
-                const double hi = (double)(a.Ns - K - O) + 1.0 + reach, lo = (double)(-O) - 1.0 - reach;
-                if (x < lo || x > hi || y < lo || y > hi) t.state = 2;
-            }
+            tp.l = (float)l;
+            tp.m = (float)m;
+            tp.n = (float)n;
+            tp.ok[2] = n2 > 0.05 + 3.0 * dmax && z > 0.05 + 3.0 * dmax && rest < 0.05;
         }
-        tp = t;
     }
     __syncthreads();
     const int qx = x0t + (threadIdx.x & (RP_TX - 1));
     if (qx >= a.Nd) return;
-    const int state = tp.state, da = qx - x0t - RP_TX / 2;
-    const float fa = (float)da;
-    const long long Xa = tp.X + da * tp.Ax, Ya = tp.Y + da * tp.Ay;
+    // 0: every pixel in FP64, 1: expansion, 2: nothing but fill
+    const int state = !(tp.ok[0] && tp.ok[1] && tp.ok[2]) ? 0 : tp.out[0] || tp.out[1] ? 2 : 1;
+    const int da = qx - x0t - RP_TX / 2;
+    const long long Xa = tp.X[0] + da * tp.A[0], Ya = tp.X[1] + da * tp.A[1];
+    const float dl = (float)da * (float)a.dl_d, n0 = tp.n;
     for (int qy = y0t + threadIdx.x / RP_TX; qy < min(y0t + RP_TY, a.Nd); qy += 256 / RP_TX) {
         const int64_t i = (int64_t)qy * a.Nd + qx;
         if (state == 2) {
@@ -211,12 +202,14 @@ __global__ void __launch_bounds__(256) reproject_kernel(ReprojArgs a) {
             continue;
         }
         const int db = qy - y0t - RP_TY / 2;
-        const float fb = (float)db;
-        const float n23 = fa * fa * (tp.q[0] + tp.q[3] * fa + tp.q[4] * fb) +
-                          fb * (tp.q[1] * fa + fb * (tp.q[2] + tp.q[5] * fa + tp.q[6] * fb));
+        const float dm = (float)db * (float)a.dl_d;
+        // n^2 = n0^2 + e1 + e2; n less its linear part = (e2 - e1 (n - n0) / (2 n0)) / (n + n0)
+        const float e1 = -2.0f * (tp.l * dl + tp.m * dm), e2 = -(dl * dl + dm * dm);
+        const float sum = sqrtf(n0 * n0 + (e1 + e2)) + n0;
+        const float rest = __fdividef(e2 - e1 * __fdividef(e1 + e2, sum * 2.0f * n0), sum);
         constexpr float ONE = (float)(1ll << RP_FRAC);
-        const long long X = Xa + db * tp.Bx + __float2ll_rn(n23 * tp.qx * ONE);
-        const long long Y = Ya + db * tp.By + __float2ll_rn(n23 * tp.qy * ONE);
+        const long long X = Xa + db * tp.B[0] + __float2ll_rn(rest * tp.rs[0] * ONE);
+        const long long Y = Ya + db * tp.B[1] + __float2ll_rn(rest * tp.rs[1] * ONE);
         const int ix = (int)(X >> RP_FRAC) + O, iy = (int)(Y >> RP_FRAC) + O;
         const uint32_t ux = (uint32_t)(X >> (RP_FRAC - 32)), uy = (uint32_t)(Y >> (RP_FRAC - 32));
         // within 2^-14 of a whole pixel with the stencil at the image's edge: FP64 decides
