@@ -779,6 +779,96 @@ __global__ void __launch_bounds__(256, NPOL == 1 ? 4 : 2) degrid_items_kernel(De
     }
 }
 
+// Stokes-I items of supports up to DGS_MAXS: one warp an item, without staging or
+// barriers.  The lanes hold the block's taps (two each) in registers and read
+// the grid for four visibilities at a time; the eight partial sums are reduced over
+// the lanes together.  A CTA an item, as above, spends such a small block's time in
+// its own latencies: 126k visibilities of 7 x 7 taps on 512^2, 25 us against 15; 8M on
+// 2048^2, 1.63 ms against 0.58.
+constexpr int DGS_MAXS = 8;
+
+template <int ST, bool SUB>
+__global__ void __launch_bounds__(256) degrid_small_kernel(DegridArgs a) {
+    constexpr int NT = DGS_MAXS * DGS_MAXS / 32;
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarps = (int64_t)gridDim.x * 8;
+    for (int64_t item = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); item < a.nitems; item += nwarps) {
+        const int4 it = a.items[item];
+        const int start = it.x, count = it.y, S = a.bin_support[it.z], L = S * S;
+        const bool mine = lane < count && AW_BOK(start + lane < a.nvalid, BC_D_REC);
+        const aw_rec r = a.rec_dg[mine ? start + lane : start];   // lane v: visibility v
+        const int64_t kb = a.bin_offset[it.z] +
+                           (int64_t)__shfl_sync(0xffffffffu, (int)r.fy * a.OS + (int)r.fx, 0) * L;
+        const uint32_t cell = (uint32_t)r.y0 * (uint32_t)a.N + r.x0;
+        float2 k[NT];
+        uint32_t off[NT];
+#pragma unroll
+        for (int i = 0; i < NT; ++i) {
+            const int t = lane + 32 * i, jy = t / S;
+            const bool on = t < L && AW_BOK(kb >= 0 && kb + L <= a.tab_elems, BC_D_SRC);
+            float2 one[1] = {make_float2(0.f, 0.f)};
+            if (on) load_k<ST, 1>(a.ktab, kb, L, t, one);
+            k[i] = one[0];
+            off[i] = on ? (uint32_t)(jy * a.N + (t - jy * S)) : 0xffffffffu;
+        }
+        for (int j = 0; j < count; j += 4) {
+            float x[8];
+            float2 g[4][NT];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t c = __shfl_sync(0xffffffffu, cell, min(j + q, count - 1));
+#pragma unroll
+                for (int i = 0; i < NT; ++i)
+                    g[q][i] = off[i] != 0xffffffffu && AW_BOK(c + off[i] < (uint32_t)a.N * (uint32_t)a.N, BC_D_GRID)
+                                  ? __ldg(a.grid + (c + off[i])) : make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float re = 0.f, im = 0.f;
+#pragma unroll
+                for (int i = 0; i < NT; ++i) {
+                    re = fmaf(k[i].x, g[q][i].x, re);
+                    re = fmaf(-k[i].y, g[q][i].y, re);
+                    im = fmaf(k[i].x, g[q][i].y, im);
+                    im = fmaf(k[i].y, g[q][i].x, im);
+                }
+                x[2 * q] = re;
+                x[2 * q + 1] = im;
+            }
+            // reduce-scatter over lane bits 4, 3, 2 (value index bits 2, 1, 0), then bits 1, 0
+#pragma unroll
+            for (int h = 4; h >= 1; h >>= 1) {
+                const bool up = lane & (4 * h);
+#pragma unroll
+                for (int i = 0; i < h; ++i) {
+                    const float send = up ? x[i] : x[i + h];
+                    const float keep = up ? x[i + h] : x[i];
+                    x[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * h);
+                }
+            }
+            x[0] += __shfl_xor_sync(0xffffffffu, x[0], 2);
+            x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
+            // lane v - j = 0 .. 3 of the four takes (re, im) from lanes 8 (v - j) and 8 (v - j) + 4
+            const float re = __shfl_sync(0xffffffffu, x[0], (lane - j) * 8 & 31);
+            const float im = __shfl_sync(0xffffffffu, x[0], ((lane - j) * 8 + 4) & 31);
+            if (mine && lane >= j && lane < j + 4 && AW_BOK(r.orig < a.nvis, BC_D_REC)) {
+                float2 o = make_float2(re * a.inv_scale, im * a.inv_scale);
+                if (r.flip) o.y = -o.y;
+                if constexpr (SUB) {
+                    const float2 w = a.sub_from[r.orig];
+                    o = make_float2(w.x - o.x, w.y - o.y);
+                }
+                a.vis_out[r.orig] = o;
+            }
+        }
+    }
+    for (int64_t i = a.nvalid + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.tail_end;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t o = (int64_t)a.rec[i].orig;
+        a.vis_out[o] = SUB ? a.sub_from[o] : make_float2(0.f, 0.f);
+    }
+}
+
 template <int NPOL, int ST>
 size_t degrid_smem_bytes() {
     constexpr bool conv = NPOL == 4 && ST != AW_STORAGE_FP32;
@@ -818,7 +908,14 @@ int launch_degrid_ts(const DegridArgs &a, int sm_count, cudaStream_t s) {
 }
 
 template <int NPOL, int ST>
-int launch_degrid_t(const DegridArgs &a, int sm_count, cudaStream_t s) {
+int launch_degrid_t(const DegridArgs &a, int max_support, int sm_count, cudaStream_t s) {
+    if (NPOL == 1 && max_support <= DGS_MAXS) {
+        const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((a.nitems + 7) / 8, (int64_t)sm_count * 8));
+        if (a.sub_from) degrid_small_kernel<ST, true><<<(unsigned)blocks, 256, 0, s>>>(a);
+        else degrid_small_kernel<ST, false><<<(unsigned)blocks, 256, 0, s>>>(a);
+        AW_CHECK_LAUNCH();
+        return AW_OK;
+    }
     return a.sub_from ? launch_degrid_ts<NPOL, ST, true>(a, sm_count, s) : launch_degrid_ts<NPOL, ST, false>(a, sm_count, s);
 }
 
@@ -959,7 +1056,7 @@ int aw_launch_degrid(const aw_plan *p, const aw_kernel_set *k, const void *grid,
     a.nvis = p->nvis;
     a.nvalid = p->nvalid;
     a.tail_end = p->nvis;
-    if (p->nitems_rgd > 0) {
+    if (p->nitems_rgd > 0 && !(p->npol == 1 && k->max_support <= DGS_MAXS)) {
         // region tasks (and the visibilities not gridded) first, the other bins here
         const int rc = aw_launch_degrid_region(p, k, grid, vis_out, s, sub_from);
         if (rc || p->nitems_ho == 0) return rc;
@@ -981,13 +1078,13 @@ int aw_launch_degrid(const aw_plan *p, const aw_kernel_set *k, const void *grid,
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int st = k->spec.storage;
     if (p->npol == 1) {
-        if (st == AW_STORAGE_FP32) return launch_degrid_t<1, AW_STORAGE_FP32>(a, sms, s);
-        if (st == AW_STORAGE_BF16) return launch_degrid_t<1, AW_STORAGE_BF16>(a, sms, s);
-        return launch_degrid_t<1, AW_STORAGE_FP16>(a, sms, s);
+        if (st == AW_STORAGE_FP32) return launch_degrid_t<1, AW_STORAGE_FP32>(a, k->max_support, sms, s);
+        if (st == AW_STORAGE_BF16) return launch_degrid_t<1, AW_STORAGE_BF16>(a, k->max_support, sms, s);
+        return launch_degrid_t<1, AW_STORAGE_FP16>(a, k->max_support, sms, s);
     }
-    if (st == AW_STORAGE_FP32) return launch_degrid_t<4, AW_STORAGE_FP32>(a, sms, s);
-    if (st == AW_STORAGE_BF16) return launch_degrid_t<4, AW_STORAGE_BF16>(a, sms, s);
-    return launch_degrid_t<4, AW_STORAGE_FP16>(a, sms, s);
+    if (st == AW_STORAGE_FP32) return launch_degrid_t<4, AW_STORAGE_FP32>(a, k->max_support, sms, s);
+    if (st == AW_STORAGE_BF16) return launch_degrid_t<4, AW_STORAGE_BF16>(a, k->max_support, sms, s);
+    return launch_degrid_t<4, AW_STORAGE_FP16>(a, k->max_support, sms, s);
 }
 
 // Bounds-check status of the kernels in this file: AW_EUNSUPPORTED unless the

@@ -521,9 +521,10 @@ struct TcDims {
     static constexpr size_t WO_OFF = 3 * (size_t)tc::TILE_BYTES;        // output layer [NOUT][LW]
     static constexpr int NWG = 3;                                       // warpgroups (tiles in flight)
     static constexpr size_t A_OFF = WO_OFF + (size_t)NOUT * LW * 2;     // one activation tile per warpgroup
-    static constexpr size_t W1_OFF = A_OFF + NWG * (size_t)tc::TILE_BYTES;  // float [LW][5]
-    static constexpr size_t B_OFF = W1_OFF + (size_t)LW * 5 * 4;        // float [4][LW] omega0 x bias, then [NOUT] bias
-    static constexpr size_t SV_OFF = (B_OFF + (size_t)(4 * LW + NOUT) * 4 + 15) / 16 * 16;
+    // layer 1, 8 floats an output (5 weights, the bias, 2 unused): two 16-byte reads
+    static constexpr size_t W1_OFF = A_OFF + NWG * (size_t)tc::TILE_BYTES;
+    static constexpr size_t B_OFF = W1_OFF + (size_t)LW * 8 * 4;        // float [3][LW] omega0 x bias, then [NOUT] bias
+    static constexpr size_t SV_OFF = (B_OFF + (size_t)(3 * LW + NOUT) * 4 + 15) / 16 * 16;
     static constexpr size_t BYTES = SV_OFF + (size_t)LCHUNK * sizeof(VisL);
 };
 
@@ -575,12 +576,12 @@ __global__ void __launch_bounds__(128 * TcDims<NPOL>::NWG, 1) grid_learned_tc_ke
         *reinterpret_cast<__half *>(sWo + tc::cm_off(o, k)) =
             (o < 2 * P) ? a.Wh[a.woff[4] + (int64_t)o * LW + k] : __float2half(0.f);
     }
-    for (int i = tid; i < LW * 5; i += blockDim.x) sW1[i] = a.Wf[a.woff[0] + i];
-    for (int i = tid; i < 4 * LW; i += blockDim.x) {
-        const float b = a.Wf[a.boff[i / LW] + (i % LW)];
-        sB[i] = (i < LW) ? b : a.omega0 * b;   // layer 1 keeps the plain bias (FP32 layer)
+    for (int i = tid; i < LW * 8; i += blockDim.x) {
+        const int o = i / 8, k = i % 8;   // layer 1 keeps the plain bias (FP32 layer)
+        sW1[i] = k < 5 ? a.Wf[a.woff[0] + o * 5 + k] : k == 5 ? a.Wf[a.boff[0] + o] : 0.f;
     }
-    for (int i = tid; i < NOUT; i += blockDim.x) sB[4 * LW + i] = (i < 2 * P) ? a.Wf[a.boff[4] + i] : 0.f;
+    for (int i = tid; i < 3 * LW; i += blockDim.x) sB[i] = a.omega0 * a.Wf[a.boff[1 + i / LW] + (i % LW)];
+    for (int i = tid; i < NOUT; i += blockDim.x) sB[3 * LW + i] = (i < 2 * P) ? a.Wf[a.boff[4] + i] : 0.f;
     if (tid == 0) {
         for (int g = 0; g < NWG; ++g) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(tc::su32(&s_mbar[g])) : "memory");
@@ -654,10 +655,13 @@ __global__ void __launch_bounds__(128 * TcDims<NPOL>::NWG, 1) grid_learned_tc_ke
                             float h[8];
 #pragma unroll
                             for (int e = 0; e < 8; ++e) {
-                                const int o = g * 8 + e;
-                                float z = sB[o];
-#pragma unroll
-                                for (int k = 0; k < 5; ++k) z = fmaf(sW1[o * 5 + k], x[k], z);
+                                const float4 wa = reinterpret_cast<const float4 *>(sW1)[2 * (g * 8 + e)];
+                                const float2 wb = reinterpret_cast<const float2 *>(sW1)[4 * (g * 8 + e) + 2];
+                                float z = fmaf(wa.x, x[0], wb.y);
+                                z = fmaf(wa.y, x[1], z);
+                                z = fmaf(wa.z, x[2], z);
+                                z = fmaf(wa.w, x[3], z);
+                                z = fmaf(wb.x, x[4], z);
                                 h[e] = __sinf(a.omega0 * z);
                             }
                             tc::st8(sA, wtid, g * 8, h);
@@ -687,7 +691,7 @@ __global__ void __launch_bounds__(128 * TcDims<NPOL>::NWG, 1) grid_learned_tc_ke
                         tc::fence_after();
                         if (!out_layer) {
                             // this row's 128 columns: omega0 (acc + bias), sine, FP16 operand
-                            const float *bw = sB + (l + 1) * LW;
+                            const float4 *bw = reinterpret_cast<const float4 *>(sB + l * LW);
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
                                 float v[32];
@@ -695,11 +699,10 @@ __global__ void __launch_bounds__(128 * TcDims<NPOL>::NWG, 1) grid_learned_tc_ke
 #pragma unroll
                                 for (int g = 0; g < 4; ++g) {
                                     float h[8];
+                                    const float4 b0 = bw[8 * q + 2 * g], b1 = bw[8 * q + 2 * g + 1];
+                                    const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-                                    for (int e = 0; e < 8; ++e) {
-                                        const int c = 32 * q + g * 8 + e;
-                                        h[e] = __sinf(fmaf(a.omega0, v[g * 8 + e], bw[c]));
-                                    }
+                                    for (int e = 0; e < 8; ++e) h[e] = __sinf(fmaf(a.omega0, v[g * 8 + e], b[e]));
                                     tc::st8(sA, wtid, 32 * q + g * 8, h);
                                 }
                             }
@@ -708,7 +711,7 @@ __global__ void __launch_bounds__(128 * TcDims<NPOL>::NWG, 1) grid_learned_tc_ke
                             float v[32];
                             tc::ld32(acc_o + lane_base, v);
 #pragma unroll
-                            for (int i = 0; i < 2 * P; ++i) kv[i] = (v[i] + sB[4 * LW + i]) * a.out_scale;
+                            for (int i = 0; i < 2 * P; ++i) kv[i] = (v[i] + sB[3 * LW + i]) * a.out_scale;
                         }
                         tc::fence_before();
                         wg_sync(wg);

@@ -671,6 +671,9 @@ static int build_hybrid_items(aw_plan *plan, cudaStream_t s) {
 // the region kernel, its tasks, and the OFFSETS items of the other bins with
 // the second stream.  The region kernel is the faster one at every support it
 // takes (aw_rg_eligible), so every plane goes there, split_planes or not.
+#ifndef RDG_MIN
+#define RDG_MIN 128
+#endif
 // The sort buffers are the plan builder's (>= nv).
 template <typename K>
 static int sort_region(aw_plan *plan, int64_t nv, const int4 *d_geo, int nb, int nt, uint64_t maxkey,
@@ -692,21 +695,35 @@ static int sort_region(aw_plan *plan, int64_t nv, const int4 *d_geo, int nb, int
     rc = build_segments<K>(keys, plan->nreg, 0, b, &nseg, s);
     if (rc == AW_OK)
         rc = build_region_tasks(nseg, plan->nreg, plan->d_rec_rg, d_geo, b, &plan->d_items_rg, &plan->nitems_rg, s);
-    if (rc == AW_OK && plan->npol == 1)
+    // region degridding pays a region's load (and its latency) per task: for tasks that
+    // are half full on average (20.16M Stokes-I visibilities, 237 a task: 2.7 against
+    // 5.7 ms; 1M, 80 a task: 472 against 357 us)
+    if (rc == AW_OK && plan->npol == 1 && plan->nreg >= (int64_t)RDG_MIN * nseg) {
         rc = build_region_tasks(nseg, plan->nreg, plan->d_rec_rg, d_geo + nb, b, &plan->d_items_rgd, &plan->nitems_rgd, s);
+        if (rc == AW_OK && plan->nreg < (int64_t)RDG_MIN * plan->nitems_rgd) plan->nitems_rgd = 0;
+    }
     return rc;
 }
 
 static int build_region(aw_plan *plan, const aw_kernel_set *ks, int64_t nv, SortBufs &b, cudaStream_t s) {
     const int nb = ks->nbins;
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // gridding geometry of every bin, then the degridding one
     std::vector<int4> geo((size_t)nb * 2, make_int4(0, 0, 0, 0));
     bool all = true;
     for (int i = 0; i < nb; ++i) {
         const int S = ks->bin_support[(size_t)i];
         if (aw_rg_eligible(S, plan->npol)) {
-            geo[(size_t)i] = make_int4(aw_rg_tile(S), AW_RG_MAXV, aw_rg_nblk(S), 0);
-            geo[(size_t)nb + i] = make_int4(aw_rg_tile(S), AW_RG_MAXV_DG, 1, 0);
+            // visibilities a task: enough tasks to fill the SMs twice (8 gridding CTAs, 6
+            // degridding CTAs each), as far as the limits allow (126k visibilities of 7 x 7 taps
+            // on 512^2: 35 us, 106 with the largest tasks)
+            const int64_t k = (int64_t)aw_rg_nblk(S) * aw_rg_nblk(S) * plan->npol;
+            const int64_t cap = std::min<int64_t>(std::max<int64_t>(nv * k / (sms * 16) / 64 * 64, 64), AW_RG_MAXV);
+            const int64_t capd = std::min<int64_t>(std::max<int64_t>(nv / (sms * 12) / 32 * 32, 32), AW_RG_MAXV_DG);
+            geo[(size_t)i] = make_int4(aw_rg_tile(S), (int)cap, aw_rg_nblk(S), 0);
+            geo[(size_t)nb + i] = make_int4(aw_rg_tile(S), (int)capd, 1, 0);
         } else {
             all = false;
         }
@@ -769,7 +786,7 @@ int aw_plan_build(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *ks, 
         return aw_set_error(AW_EINVAL, "vis descriptor incomplete");
     if (vis->nvis > 0x7fffffffLL) return aw_set_error(AW_EINVAL, "nvis %lld above 2^31-1", (long long)vis->nvis);
     const aw_kernel_spec &sp = ks->spec;
-    aw_tune t = tune ? *tune : aw_tune{32, 256, 2, 0, AW_GRID_TILES};
+    aw_tune t = tune ? *tune : aw_tune{32, 256, 5, 0, AW_GRID_TILES};
     if (t.tile < 8 || t.tile > 256 || (t.tile & (t.tile - 1))) return aw_set_error(AW_EINVAL, "tile %d", t.tile);
     if (t.chunk < 32 || t.chunk > 2048) return aw_set_error(AW_EINVAL, "chunk %d", t.chunk);
     if (t.ctas_per_sm < 1 || t.ctas_per_sm > 8) t.ctas_per_sm = 2;
