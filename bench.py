@@ -316,11 +316,8 @@ def wproj_section(ctx, dev, args, stream):
              "offsets": aw.aw_tune(32, 256, 4, 256, aw.AW_GRID_OFFSETS, 0),
              "hybrid/16": aw.aw_tune(32, 256, 2, 256, aw.AW_GRID_HYBRID, 16),
              "hybrid/24": aw.aw_tune(32, 256, 2, 256, aw.AW_GRID_HYBRID, 24),
-             # the region kernel for supports 16-48 (8 and wider on OFFSETS beside it)
-             "region": aw.aw_tune(32, 256, 2, 1024, aw.AW_GRID_REGION, 0),
-             "region/14": aw.aw_tune(32, 256, 2, 1024, aw.AW_GRID_REGION, 14),
-             "region/18": aw.aw_tune(32, 256, 2, 1024, aw.AW_GRID_REGION, 18),
-             "region/22": aw.aw_tune(32, 256, 2, 1024, aw.AW_GRID_REGION, 22)}
+             # the region kernel for supports 8-48 (the wider ones on OFFSETS beside it)
+             "region": aw.aw_tune(32, 256, 2, 1024, aw.AW_GRID_REGION, 0)}
 
     def ms_of(fn, reps=5):
         fn()
@@ -992,8 +989,7 @@ def learned_degrid(ctx, dev, args, kw, kw_fine, vd, obs, stream, timed, kmax, ch
 # ----------------------------------------------------------------------------- GPU arm
 def wproj_case(reps: int):
     """Configuration 2 for profiling: 20.16M Stokes-I visibilities, 2048^2, 32 w planes (supports 8-64),
-    OS 8, FP32 tables; the region schedule with planes 0-17 on the region kernel (the bench's choice for
-    this configuration); one untimed grid + degrid, then `reps` timed ones."""
+    OS 8, FP32 tables; the region schedule (the bench's choice for this configuration); one untimed grid + degrid, then `reps` timed ones."""
     import torch
     from paper_2206_15117_gb300 import aw
     from paper_2206_15117_gb300 import build as awbuild
@@ -1007,7 +1003,7 @@ def wproj_case(reps: int):
     kg = aw.aw_make_kernels(ctx, **kw, role=aw.AW_ROLE_GRID)
     kd = aw.aw_make_kernels(ctx, **kw, role=aw.AW_ROLE_DEGRID)
     vd, keep = aw.device_observation(ob, dev)
-    plan = aw.aw_plan_create(ctx, vd, kg, tune=aw.aw_tune(32, 256, 2, 1024, aw.AW_GRID_REGION, 18))
+    plan = aw.aw_plan_create(ctx, vd, kg, tune=aw.aw_tune(32, 256, 2, 1024, aw.AW_GRID_REGION, 0))
     gen = torch.Generator(device=dev)
     gen.manual_seed(2)
     vis = torch.randn((ob.nvis, 1), dtype=torch.complex64, device=dev, generator=gen)
@@ -1154,11 +1150,7 @@ def run_ours(args, rank, world, dist):
         for share in (0.25, 0.30, 0.35, 0.40):
             finalists.append(aw.aw_tune(tune.tile, tune.chunk, 2, 1024, aw.AW_GRID_HYBRID,
                                         hybrid_split(aw, plan, kw, share)))
-        # the region schedule with the planes of supports up to 32, 40 and 48 cells on the region kernel
-        for lim in (32, 40, 48):
-            q = sum(1 for s_ in kw["supports"] if s_ <= lim)
-            if 0 < q:
-                finalists.append(aw.aw_tune(tune.tile, tune.chunk, 2, 1024, aw.AW_GRID_REGION, q))
+        finalists.append(aw.aw_tune(tune.tile, tune.chunk, 2, 1024, aw.AW_GRID_REGION, kw["nw"]))
         key = lambda t_: (t_.grid_mode, t_.ctas_per_sm if t_.grid_mode != aw.AW_GRID_OFFSETS else 0,
                           t_.split_planes if t_.grid_mode in (aw.AW_GRID_HYBRID, aw.AW_GRID_REGION) else 0,
                           t_.dg_tile or 1024)
@@ -1522,7 +1514,7 @@ TRAFFIC_PER_VIS = {"region": 146.5e6 / 1139896, "degrid_items_kernel": 96.5e6 / 
 def roofline_entry(kernel, achieved, peak, peak_src, flops, g_ms, d_ms, region, nvalid, subset):
     """The `roofline` object of the dominant step (gridding if g_ms >= d_ms).  `traffic` is the
     scaled one-bin-pair capture when it describes the kernel that runs: the degridder; the region
-    capture predates the region kernel's three-pass units (supports 20 and 24), so for the region
+    capture predates the present region kernel (one plane a CTA), so for the region
     schedule `traffic` is null and the previous figure stands beside it, labelled.  Null at the
     subset scale and for the other schedules."""
     traffic, traffic_prev = None, None
@@ -1539,8 +1531,8 @@ def roofline_entry(kernel, achieved, peak, peak_src, flops, g_ms, d_ms, region, 
     if traffic_prev:
         roof["traffic_previous_region_kernel"] = {
             "bytes": traffic_prev,
-            "source": "profiles/dram_traffic_fullpol_aw_1pair.md (the region kernel with paired passes, before "
-                      "the three-pass units), scaled by the visibility count (lower bound)"}
+            "source": "profiles/dram_traffic_fullpol_aw_1pair.md (the former region kernel, four planes a CTA), "
+                      "scaled by the visibility count (lower bound)"}
     return roof
 
 

@@ -553,7 +553,7 @@ int aw_autotune(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *k, aw_
     // OFFSETS, its super-tile the larger one)
     bool any_region = false;
     for (int32_t S : k->bin_support) any_region = any_region || aw_rg_eligible(S, k->spec.npol);
-    if (!rc && any_region) {
+    if (!rc && any_region && k->max_support > AW_RG_MIN_SUPPORT) {
         aw_tune tu{bt.tile, bt.chunk, 2, 1024, AW_GRID_REGION, k->spec.nw};
         aw_plan *p = new aw_plan();
         p->device = ctx->device;

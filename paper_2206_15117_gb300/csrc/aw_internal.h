@@ -212,14 +212,17 @@ __host__ __device__ inline int aw_rg_tile(int S) {
     return AW_RG_R + 1 - (S <= 8 ? 8 : aw_rg_n24(S) ? 24 : 16);
 }
 // Supports on the region kernels: padding the footprint to a multiple of 8 taps
-// a side costs at most 1.8 times the taps (about what OFFSETS costs more), and a
-// block of 8 x 8 taps is left to OFFSETS where it gives a thread too little to do
-// (300k full-pol visibilities of 8 x 8 taps: 149 us against 189; 126k of 7 x 7 in
-// Stokes I: 29 against 35).  Stokes I: up to 48 cells (wider ones hold few
-// visibilities a tile).
+// a side costs at most 1.8 times the taps (about what OFFSETS costs more).
+// Stokes I: up to 48 cells (wider ones hold few visibilities a tile).  A set with
+// no support above AW_RG_MIN_SUPPORT stays on OFFSETS: blocks of 8 x 8 taps alone
+// give the region kernel too little to do between its barriers (300k full-pol
+// visibilities of 8 x 8 taps: 149 us against 189; 126k of 7 x 7 in Stokes I: 29
+// against 35), beside wider ones they are better off there than on OFFSETS' one CTA
+// per SM (3M with supports 8-64: 5.0 ms against 6.3).
+constexpr int AW_RG_MIN_SUPPORT = 8;
 inline bool aw_rg_eligible(int S, int npol) {
     const int p = (S + 7) / 8 * 8;
-    return S >= (npol == 1 ? 8 : 9) && S <= (npol == 1 ? 48 : 128) && 10 * p * p <= 18 * S * S;
+    return S >= 2 && S <= (npol == 1 ? 48 : 128) && 10 * p * p <= 18 * S * S;
 }
 // task word: tile column and row (9 bits each: at most 16384 / 33), block column and row (3 bits each)
 __host__ __device__ inline int aw_rg_pack(int tx, int ty, int bx, int by) {

@@ -451,18 +451,35 @@ __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::be
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void fence_smem_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
-__device__ __forceinline__ void ld32(uint32_t taddr, float (&v)[32]) {
-    uint32_t r[32];
+// 32 columns of the thread's accumulator row: the load, and the wait that makes
+// every earlier load's registers valid (they pass through it, so that no use moves
+// ahead of it)
+__device__ __forceinline__ void ld32_start(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
         "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]),
+          "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
+          "=r"(r[30]), "=r"(r[31])
         : "r"(taddr)
         : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void ld32_wait(uint32_t (&r)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                   "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]),
+                   "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]),
+                   "+r"(r[30]), "+r"(r[31])
+                 :
+                 : "memory");
+}
+__device__ __forceinline__ void ld32(uint32_t taddr, float (&v)[32]) {
+    uint32_t r[32];
+    ld32_start(taddr, r);
+    ld32_wait(r);
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
@@ -692,17 +709,21 @@ __global__ void __launch_bounds__(128 * TcDims<NPOL>::NWG, 1) grid_learned_tc_ke
                         if (!out_layer) {
                             // this row's 128 columns: omega0 (acc + bias), sine, FP16 operand
                             const float4 *bw = reinterpret_cast<const float4 *>(sB + l * LW);
+// the next 32 columns load while these are worked on
+                            uint32_t r[2][32];
+                            tc::ld32_start(acc_h + lane_base, r[0]);
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
-                                float v[32];
-                                tc::ld32(acc_h + lane_base + 32 * q, v);
+                                tc::ld32_wait(r[q & 1]);
+                                if (q < 3) tc::ld32_start(acc_h + lane_base + 32 * (q + 1), r[(q + 1) & 1]);
 #pragma unroll
                                 for (int g = 0; g < 4; ++g) {
                                     float h[8];
                                     const float4 b0 = bw[8 * q + 2 * g], b1 = bw[8 * q + 2 * g + 1];
                                     const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-                                    for (int e = 0; e < 8; ++e) h[e] = __sinf(fmaf(a.omega0, v[g * 8 + e], b[e]));
+                                    for (int e = 0; e < 8; ++e)
+                                        h[e] = __sinf(fmaf(a.omega0, __uint_as_float(r[q & 1][g * 8 + e]), b[e]));
                                     tc::st8(sA, wtid, 32 * q + g * 8, h);
                                 }
                             }

@@ -31,6 +31,7 @@ struct ReprojArgs {
     double dl_d, cx_d, cy_d;     // destination frame
     double inv_dl_s, cx_s, cy_s; // source frame
     int Nd, Ns, nplane;
+    int ty;                      // rows of a destination tile
     float fill;
 };
 
@@ -114,7 +115,7 @@ __device__ __noinline__ void reproject_pixel64(const ReprojArgs &a, int qx, int 
 // fixed point with RP_FRAC fraction bits: X + a A + b B is exact in the direction
 // cosines l, m and linear in n = sqrt(1 - l^2 - m^2); the rest of n is added in FP32.
 constexpr int RP_FRAC = 40;
-constexpr int RP_TX = 64, RP_TY = 32;
+constexpr int RP_TX = 64;
 struct TilePos {
     long long X[2], A[2], B[2];   // x and y: at the centre, per column, per row
     float rs[2];                  // R[2], R[5] over the source pixel size
@@ -122,7 +123,7 @@ struct TilePos {
     int ok[3], out[2];
 };
 
-// A CTA takes a tile of 64 x 32 destination pixels.  FP64 is slow on this part:
+// A CTA takes a tile of 64 x TY destination pixels.  FP64 is slow on this part:
 // the position map is expanded about the tile centre in FP64 once and evaluated
 // for the pixels in 64-bit integers.  What n departs from its linear part by comes
 // from the difference of squares, with no cancellation, so FP32 gives it to a few
@@ -131,46 +132,46 @@ struct TilePos {
 // interpolation weights.  Where a position lies so close to a whole pixel that its
 // rounding could decide whether the stencil is inside the image, the pixel is done
 // in FP64.  Seven fields of 2048^2 x 4 onto 4096^2 x 4 with their weights and
-// combination: 5.37 -> 1.66 ms; one field 620 -> 158 us, of 256^2 onto 400^2
-// 17.1 -> 16.7 us.
+// combination: 5.37 -> RP_MS ms; one field 620 -> RP_BIG us, of 256^2 onto 400^2
+// 17.1 -> RP_SMALL us.
 template <int INTERP>
 __global__ void __launch_bounds__(256) reproject_kernel(ReprojArgs a) {
     constexpr int K = (INTERP == AW_INTERP_CUBIC) ? 4 : 2;
     constexpr int O = (INTERP == AW_INTERP_CUBIC) ? -1 : 0;
     __shared__ TilePos tp;
-    const int x0t = blockIdx.x * RP_TX, y0t = blockIdx.y * RP_TY;
-    // the lead lanes of three warps share the FP64 work: a small image waits for its latency
-    const int role = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0 && role < 3) {
+    const int TY = a.ty, x0t = blockIdx.x * RP_TX, y0t = blockIdx.y * TY;
+    // three lanes: x, y and the third direction cosine (a warp's FP64 instruction takes the
+    // same time for one lane as for all, and a small image waits for its latency)
+    if (threadIdx.x < 3) {
+        const int i = threadIdx.x;
         const double l = ((double)(x0t + RP_TX / 2) - a.cx_d) * a.dl_d;
-        const double m = ((double)(y0t + RP_TY / 2) - a.cy_d) * a.dl_d;
+        const double m = ((double)(y0t + TY / 2) - a.cy_d) * a.dl_d;
         const double n2 = 1.0 - l * l - m * m;
         const double i1 = rsqrt(fmax(n2, 0.05)), n = n2 * i1;   // (used for n^2 > 0.05 only)
-        const double s = a.inv_dl_s;
-        if (role < 2) {
-            // x or y at the centre and its slopes
-            const double r0 = a.R[3 * role], r1 = a.R[3 * role + 1], r2 = a.R[3 * role + 2];
-            const double ds = a.dl_d * s;
-            const double x = (r0 * l + r1 * m + r2 * n) * s + (role ? a.cy_s : a.cx_s);
-            const double ax = (r0 - r2 * (l * i1)) * ds, bx = (r1 - r2 * (m * i1)) * ds;
-            const double reach = 64.0 * fmax(fabs(ax), fabs(bx)) + 4.0;
-            const bool ok = reach < 4096.0 && fabs(x) < 4.0e6;
+        const double r0 = a.R[3 * i], r1 = a.R[3 * i + 1], r2 = a.R[3 * i + 2];
+        const double s = i < 2 ? a.inv_dl_s : 1.0, ds = a.dl_d * s;
+        const double x = (r0 * l + r1 * m + r2 * n) * s + (i == 0 ? a.cx_s : i == 1 ? a.cy_s : 0.0);
+        const double sx = (r0 - r2 * (l * i1)) * ds, sy = (r1 - r2 * (m * i1)) * ds;
+        const float xf = (float)x, nf = (float)n;
+        const float reach = 64.0f * fmaxf(fabsf((float)sx), fabsf((float)sy)) + 4.0f;
+        // dmax: the farthest offset in the tile, at most sqrt(32^2 + 32^2) pixels
+        const float dmax = (float)a.dl_d * 46.0f;
+        if (i < 2) {
+            const bool ok = reach < 4096.0f && fabsf(xf) < 4.0e6f &&
+                            2.0f * dmax * dmax / (nf * nf * nf) * fabsf((float)(r2 * s)) < 0.05f;
             const double one = (double)(1ll << RP_FRAC);
-            tp.X[role] = ok ? llrint(x * one) : 0;
-            tp.A[role] = ok ? llrint(ax * one) : 0;
-            tp.B[role] = ok ? llrint(bx * one) : 0;
-            tp.rs[role] = (float)(r2 * s);
-            tp.ok[role] = ok;
+            tp.X[i] = ok ? llrint(x * one) : 0;
+            tp.A[i] = ok ? llrint(sx * one) : 0;
+            tp.B[i] = ok ? llrint(sy * one) : 0;
+            tp.rs[i] = (float)(r2 * s);
+            tp.ok[i] = ok;
             // every stencil of the tile well outside the image
-            tp.out[role] = x < (double)(-O) - 1.0 - reach || x > (double)(a.Ns - K - O) + 1.0 + reach;
+            tp.out[i] = xf < (float)(-O) - 2.0f - reach || xf > (float)(a.Ns - K - O) + 2.0f + reach;
         } else {
-            const double dmax = a.dl_d * 36.0;   // farthest offset in the tile: sqrt(32^2 + 16^2) = 35.8
-            const double rest = 2.0 * dmax * dmax * (i1 * i1) * i1 * s * fmax(fabs(a.R[2]), fabs(a.R[5]));
-            const double z = a.R[6] * l + a.R[7] * m + a.R[8] * n;
             tp.l = (float)l;
             tp.m = (float)m;
-            tp.n = (float)n;
-            tp.ok[2] = n2 > 0.05 + 3.0 * dmax && z > 0.05 + 3.0 * dmax && rest < 0.05;
+            tp.n = nf;
+            tp.ok[2] = (float)n2 > 0.05f + 3.0f * dmax && xf > 0.05f + 3.0f * dmax;
         }
     }
     __syncthreads();
@@ -181,7 +182,7 @@ __global__ void __launch_bounds__(256) reproject_kernel(ReprojArgs a) {
     const int da = qx - x0t - RP_TX / 2;
     const long long Xa = tp.X[0] + da * tp.A[0], Ya = tp.X[1] + da * tp.A[1];
     const float dl = (float)da * (float)a.dl_d, n0 = tp.n;
-    for (int qy = y0t + threadIdx.x / RP_TX; qy < min(y0t + RP_TY, a.Nd); qy += 256 / RP_TX) {
+    for (int qy = y0t + threadIdx.x / RP_TX; qy < min(y0t + TY, a.Nd); qy += 256 / RP_TX) {
         const int64_t i = (int64_t)qy * a.Nd + qx;
         if (state == 2) {
             fill_pixel(a, i);
@@ -201,7 +202,7 @@ __global__ void __launch_bounds__(256) reproject_kernel(ReprojArgs a) {
             else reproject_pixel64<INTERP>(a, qx, qy);
             continue;
         }
-        const int db = qy - y0t - RP_TY / 2;
+        const int db = qy - y0t - TY / 2;
         const float dm = (float)db * (float)a.dl_d;
         // n^2 = n0^2 + e1 + e2; n less its linear part = (e2 - e1 (n - n0) / (2 n0)) / (n + n0)
         const float e1 = -2.0f * (tp.l * dl + tp.m * dm), e2 = -(dl * dl + dm * dm);
@@ -369,7 +370,9 @@ int aw_reproject(aw_ctx *ctx, const float *src, const aw_sky_frame *sf, float *d
     a.nplane = nplane;
     a.fill = fill;
     cudaStream_t s = S_(stream);
-    const dim3 tiles((df->N + RP_TX - 1) / RP_TX, (df->N + RP_TY - 1) / RP_TY);
+    // tall tiles share the FP64 work, low ones spread a small image over the SMs
+    a.ty = df->N >= 2048 ? 64 : df->N >= 1024 ? 32 : 8;
+    const dim3 tiles((df->N + RP_TX - 1) / RP_TX, (df->N + a.ty - 1) / a.ty);
     if (interp == AW_INTERP_CUBIC)
         reproject_kernel<AW_INTERP_CUBIC><<<tiles, 256, 0, s>>>(a);
     else

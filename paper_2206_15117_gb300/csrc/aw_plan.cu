@@ -715,7 +715,7 @@ static int build_region(aw_plan *plan, const aw_kernel_set *ks, int64_t nv, Sort
     bool all = true;
     for (int i = 0; i < nb; ++i) {
         const int S = ks->bin_support[(size_t)i];
-        if (aw_rg_eligible(S, plan->npol)) {
+        if (ks->max_support > AW_RG_MIN_SUPPORT && aw_rg_eligible(S, plan->npol)) {
             // visibilities a task: enough tasks to fill the SMs twice (8 gridding CTAs, 6
             // degridding CTAs each), as far as the limits allow (126k visibilities of 7 x 7 taps
             // on 512^2: 35 us, 106 with the largest tasks)
