@@ -784,8 +784,11 @@ __global__ void __launch_bounds__(256, NPOL == 1 ? 4 : 2) degrid_items_kernel(De
 // the grid for four visibilities at a time; the eight partial sums are reduced over
 // the lanes together.  A CTA an item, as above, spends such a small block's time in
 // its own latencies: 126k visibilities of 7 x 7 taps on 512^2, 25 us against 15; 8M on
-// 2048^2, 1.63 ms against 0.58.
+// 2048^2, 1.63 ms against 0.58.  Below DGS_MIN visibilities the SMs have a few items
+// each and the warp's serial walk through its item is the whole time: 23k
+// visibilities 8.6 us by CTAs against 14.6, 36k 15.0 / 17.1, 76k 16.7 / 14.6.
 constexpr int DGS_MAXS = 8;
+constexpr int64_t DGS_MIN = 65536;
 
 template <int ST, bool SUB>
 __global__ void __launch_bounds__(256) degrid_small_kernel(DegridArgs a) {
@@ -909,7 +912,7 @@ int launch_degrid_ts(const DegridArgs &a, int sm_count, cudaStream_t s) {
 
 template <int NPOL, int ST>
 int launch_degrid_t(const DegridArgs &a, int max_support, int sm_count, cudaStream_t s) {
-    if (NPOL == 1 && max_support <= DGS_MAXS) {
+    if (NPOL == 1 && max_support <= DGS_MAXS && a.nvalid >= DGS_MIN) {
         const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((a.nitems + 7) / 8, (int64_t)sm_count * 8));
         if (a.sub_from) degrid_small_kernel<ST, true><<<(unsigned)blocks, 256, 0, s>>>(a);
         else degrid_small_kernel<ST, false><<<(unsigned)blocks, 256, 0, s>>>(a);

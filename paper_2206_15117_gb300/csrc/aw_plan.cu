@@ -781,7 +781,6 @@ int aw_plan_plane_taps(const aw_plan *plan, std::vector<double> &cum, cudaStream
 
 int aw_plan_build(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *ks, const aw_tune *tune,
                   aw_plan *plan, cudaStream_t s) {
-    (void)ctx;
     if (!vis || vis->nvis < 0 || (vis->nvis > 0 && (!vis->uvw || !vis->row_of_vis || !vis->chan_of_vis || !vis->freq)))
         return aw_set_error(AW_EINVAL, "vis descriptor incomplete");
     if (vis->nvis > 0x7fffffffLL) return aw_set_error(AW_EINVAL, "nvis %lld above 2^31-1", (long long)vis->nvis);
@@ -899,6 +898,12 @@ int aw_plan_build(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *ks, 
     int rc = kbits <= 32 ? grid_order(uint32_t()) : grid_order(uint64_t());
     if (rc || plan->nvalid == 0) return rc;
     const int64_t nv = plan->nvalid;
+    // CTAs an SM of the default schedule: five for Stokes I (5083 items 125 us against 179
+    // with two, 353 items 27.3 / 27.3).  At full polarisation they meet on the cells of
+    // the few tiles that are in work, so three (9815 items 2.69 ms against 3.06; five 2.69) and
+    // two for small sets (490 items 70.7 us against 75.3 with three and 78.5 with five, 624
+    // items 59.3 / 64.2 / 67.5, 1222 items equal, 1297 items 427 / 360 / 342).
+    if (!tune && plan->npol == 4) plan->tune.ctas_per_sm = plan->nitems >= 8 * (int64_t)ctx->sm_count ? 3 : 2;
 
     // degridding order: (bin, super-tile, oversampled offset), the grid order inside
     const int stbits = ilog2(plan->dg_tile);

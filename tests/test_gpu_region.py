@@ -64,3 +64,21 @@ def test_region_padded_support_reduced_precision(ctx, storage, tol):
     assert l2 < tol and mx < 4 * tol, (l2, mx)
     l2, _ = rel_err(c.gpu_degrid(), c.oracle_degrid())
     assert l2 < tol, l2
+
+
+# supports of at most 8 (one warp an item from 65536 visibilities, a CTA an item
+# below); the subtraction adds one FP32 rounding to the prediction
+@pytest.mark.parametrize("n_t", [200, 300])
+def test_degrid_small_supports(ctx, n_t):
+    import torch
+    from paper_2206_15117_gb300 import aw
+    ob, kw = _stokes_i((7, 8), n_t=n_t)
+    flags = (np.random.default_rng(6).random(ob.nvis) < 0.05).astype(np.uint8)
+    c = Case(ctx, ob, kw, tune=aw.aw_tune(32, 256, 2, 256, 1), flags=flags)
+    assert (int((c.co.valid == 1).sum()) >= 65536) == (n_t == 300)
+    _check_degrid(c)
+    vis, out = torch.as_tensor(c.vis, device="cuda"), torch.zeros_like(torch.as_tensor(c.vis, device="cuda"))
+    aw.aw_degrid_subtract(ctx, c.plan, c.kd, torch.as_tensor(c.model, device="cuda"), vis, out)
+    pred = c.gpu_degrid()
+    eps = 2.0 ** -23 * (np.abs(c.vis).max() + np.abs(pred).max())
+    assert np.abs(out.cpu().numpy() - (c.vis - pred)).max() <= 2 * eps
