@@ -385,8 +385,8 @@ int aw_autotune(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *kset, 
  * are written as 0.  grid (device complex64 [npol][N][N], kset's N and npol)
  * is used as FFT scratch and left transformed (the plain unscaled inverse FFT);
  * image: device float
- * [npol][N][N].  cuFFT (FP32 complex) plus the library's own shift and
- * grid-correction kernels.
+ * [npol][N][N].  FP32 complex: the library's own two-pass transform for N = 256
+ * to 4096, cuFFT and a grid-correction kernel otherwise.
  */
 int aw_fft_to_image(aw_ctx *ctx, const aw_kernel_set *kset, void *grid, double weight_sum,
                     float *image, void *stream);

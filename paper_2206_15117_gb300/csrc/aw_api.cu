@@ -118,6 +118,7 @@ int aw_destroy(aw_ctx *ctx) {
     use_device(ctx->device);
     for (auto &kv : ctx->fft_plans) cufftDestroy(kv.second);
     for (auto &kv : ctx->gridcorr) aw_dev_free(kv.second);
+    for (auto &kv : ctx->twiddle) aw_dev_free(kv.second);
     if (ctx->d_scratch) aw_dev_free(ctx->d_scratch);
     delete ctx;
     return AW_OK;

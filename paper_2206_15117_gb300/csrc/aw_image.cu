@@ -9,7 +9,8 @@ namespace {
 // The centring phases (-1)^(x + y) of both sides of a transform: those of one
 // side are a shift of the other side by N/2 on each axis (N a multiple of 4), so
 // they are applied as signs on the image side and as a shifted position, also on
-// the image side, and the grid needs no pass of its own.  A CTA works on one
+// the image side, and the grid needs no pass of its own.  The kernels here are for
+// the N that have no transform of the library's own.  A CTA works on one
 // row of one plane (blockIdx.y, blockIdx.z), a thread on V pixels of it; V = 4
 // for arrays aligned to 16 bytes.
 
@@ -181,15 +182,16 @@ int aw_fft_to_image_impl(aw_ctx *ctx, int N, int npol, double W, void *grid, dou
     float *corr = nullptr;
     int rc = aw_ctx_gridcorr(ctx, N, W, &corr);
     if (rc) return rc;
+    float2 *g = reinterpret_cast<float2 *>(grid);
+    const float inv = (float)(1.0 / weight_sum);
+    if (aw_fft_has(N)) return aw_fft_grid_to_image(ctx, N, npol, g, corr, inv, image, s);
     cufftHandle plan;
     rc = aw_ctx_fft_plan(ctx, 2, N, npol, CUFFT_C2C, &plan);
     if (rc) return rc;
     AW_CUFFT_TRY(cufftSetStream(plan, s));
-    float2 *g = reinterpret_cast<float2 *>(grid);
     AW_CUFFT_TRY(cufftExecC2C(plan, reinterpret_cast<cufftComplex *>(g), reinterpret_cast<cufftComplex *>(g),
                               CUFFT_INVERSE));
     dim3 nb, nt;
-    const float inv = (float)(1.0 / weight_sum);
     if (aligned16(g, image)) {
         row_shape(N, npol, 4, nb, nt);
         gridcorr_kernel<4><<<nb, nt, 0, s>>>(g, corr, N, inv, image);
@@ -210,11 +212,12 @@ int aw_image_to_grid_impl(aw_ctx *ctx, int N, int npol, double W, const float *i
     float *corr = nullptr;
     int rc = aw_ctx_gridcorr(ctx, N, W, &corr);
     if (rc) return rc;
+    float2 *g = reinterpret_cast<float2 *>(grid);
+    if (aw_fft_has(N)) return aw_fft_image_to_grid(ctx, N, npol, image, corr, g, s);
     cufftHandle plan;
     rc = aw_ctx_fft_plan(ctx, 2, N, npol, CUFFT_C2C, &plan);
     if (rc) return rc;
     AW_CUFFT_TRY(cufftSetStream(plan, s));
-    float2 *g = reinterpret_cast<float2 *>(grid);
     dim3 nb, nt;
     if (aligned16(g, image)) {
         row_shape(N, npol, 4, nb, nt);

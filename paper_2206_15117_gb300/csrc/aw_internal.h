@@ -70,6 +70,8 @@ struct aw_ctx {
     std::map<std::tuple<int, int, int, int>, cufftHandle> fft_plans;
     // grid-correction vectors keyed by (N, W)
     std::map<std::pair<int, double>, float *> gridcorr;
+    // twiddle factors of the library's own transforms, by N
+    std::map<int, float2 *> twiddle;
     // small device scratch: [0] reduction word for mosaic_gamma
     unsigned int *d_scratch = nullptr;
     // last aw_autotune result (used by aw_plan_create when given no tune)
@@ -290,6 +292,12 @@ int aw_degrid_region_bounds_status(unsigned int *v, int reset);
 int aw_plan_plane_taps(const aw_plan *plan, std::vector<double> &cum, cudaStream_t s);
 int aw_launch_degrid(const aw_plan *plan, const aw_kernel_set *kset, const void *grid,
                      void *vis_out, cudaStream_t stream, const void *sub_from = nullptr);
+// The library's own two-pass transforms (aw_fft.cu), for the N that it has.
+bool aw_fft_has(int N);
+int aw_fft_grid_to_image(aw_ctx *ctx, int N, int npol, float2 *g, const float *corr, float inv_wsum, float *image,
+                         cudaStream_t s);
+int aw_fft_image_to_grid(aw_ctx *ctx, int N, int npol, const float *image, const float *corr, float2 *g,
+                         cudaStream_t s);
 int aw_fft_to_image_impl(aw_ctx *ctx, int N, int npol, double W, void *grid, double weight_sum,
                          float *image, cudaStream_t s);
 int aw_image_to_grid_impl(aw_ctx *ctx, int N, int npol, double W, const float *image, void *grid,
