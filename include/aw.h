@@ -175,8 +175,8 @@ typedef struct aw_tune {
  * visibilities of an offset, and adds the region to the grid once; bins whose
  * support has no region form (padded to a multiple of 8 taps a side it would
  * cost more than 1.8 times the taps; Stokes I: above 48 cells; every support 8 or
- * less) take OFFSETS on
- * the plan's second stream at the same time.  split_planes is checked (0..nw)
+ * less) take OFFSETS on the plan's second stream at the same time, and a full-pol
+ * set with fewer than 24 visibilities a bin and region tile takes OFFSETS alone.  split_planes is checked (0..nw)
  * but does not move planes to OFFSETS, which is the slower one at every
  * support with a region form.  All modes give the same grid up to FP32
  * rounding order. */

@@ -674,6 +674,12 @@ static int build_hybrid_items(aw_plan *plan, cudaStream_t s) {
 #ifndef RDG_MIN
 #define RDG_MIN 128
 #endif
+// Sparse full-pol sets take OFFSETS alone: below RG_SPARSE visibilities a bin and
+// region tile, clearing and adding the four planes of a region costs more than
+// atomics (25k visibilities of 128 bins on 4096^2, 4 a tile: 506 us against 173; 45 sets of
+// 20k-2.9M: OFFSETS the faster one in all 26 below 28, equal about 60, up to 0.55 of
+// its speed above 200).
+constexpr int64_t RG_SPARSE = 24;
 // The sort buffers are the plan builder's (>= nv).
 template <typename K>
 static int sort_region(aw_plan *plan, int64_t nv, const int4 *d_geo, int nb, int nt, uint64_t maxkey,
@@ -693,6 +699,10 @@ static int sort_region(aw_plan *plan, int64_t nv, const int4 *d_geo, int nb, int
     AW_CHECK_LAUNCH();
     int64_t nseg = 0;
     rc = build_segments<K>(keys, plan->nreg, 0, b, &nseg, s);
+    if (rc == AW_OK && plan->npol == 4 && plan->nreg < RG_SPARSE * nseg) {
+        plan->nreg = 0;
+        return AW_OK;
+    }
     if (rc == AW_OK)
         rc = build_region_tasks(nseg, plan->nreg, plan->d_rec_rg, d_geo, b, &plan->d_items_rg, &plan->nitems_rg, s);
     // region degridding pays a region's load (and its latency) per task: for tasks that
@@ -740,6 +750,10 @@ static int build_region(aw_plan *plan, const aw_kernel_set *ks, int64_t nv, Sort
     const int rc = key_bits(maxkey) <= 32 ? sort_region<uint32_t>(plan, nv, d_geo, nb, nt, maxkey, d_nreg, b, s)
                                           : sort_region<uint64_t>(plan, nv, d_geo, nb, nt, maxkey, d_nreg, b, s);
     if (rc) return rc;
+    if (plan->nreg == 0) {
+        all = false;
+        std::fill(geo.begin(), geo.end(), make_int4(0, 0, 0, 0));
+    }
     // the other bins: their degridding items on the OFFSETS schedule
     if (!all) {
         std::vector<int4> hd((size_t)plan->nitems_dg), keep;

@@ -82,3 +82,15 @@ def test_degrid_small_supports(ctx, n_t):
     pred = c.gpu_degrid()
     eps = 2.0 ** -23 * (np.abs(c.vis).max() + np.abs(pred).max())
     assert np.abs(out.cpu().numpy() - (c.vis - pred)).max() <= 2 * eps
+
+
+# full-pol sets with few visibilities a bin and tile take OFFSETS alone
+def test_sparse_set_takes_offsets(ctx):
+    from paper_2206_15117_gb300 import aw
+    ob, kw = case_fullpol(supports=(24, 32, 40), n_t=1, radius=200.0)
+    c = Case(ctx, ob, kw, tune=aw.aw_tune(32, 256, 2, 256, REGION))
+    info = aw.aw_plan_query(c.plan)
+    assert info.region_lists == 0 and info.grid_kernels == 1
+    _check_grid(c)
+    _check_grid(c, batched=True)
+    _check_degrid(c)
