@@ -25,9 +25,9 @@
 // visibility-tap and plane plus the kernel loads of every run; at full
 // polarisation the FP32 pipe has the same limit of 0.5 clocks per
 // visibility-tap.  Measured on 12M full-pol visibilities at 4096^2 (supports
-// 16-72): 25.8 ms (the pipe 79 % busy) against 34.9 ms for the former form, four
+// 16-72): 24.9 ms (the pipe 79 % busy) against 34.3 ms for the former form, four
 // planes a CTA with the warps kept apart by footprint-row residues and OFFSETS
-// beside it; 20.16M Stokes-I visibilities at 2048^2: 4.0 against 7.4 ms.  One
+// beside it; 20.16M Stokes-I visibilities at 2048^2: 3.5 against 6.8 ms.  One
 // warp a region was slower (29.6 ms: two warps a scheduler do not hide their
 // own latencies), and so was loading the next run's kernel values into a second
 // register set (36-45 ms).
