@@ -132,7 +132,8 @@ typedef struct aw_vis_desc {
     const double *uvw;          /* device f64 [nrow][3], metres                  */
     const uint32_t *row_of_vis; /* device [nvis]                                 */
     const uint16_t *chan_of_vis;/* device [nvis]                                 */
-    const double *freq;         /* device f64 [nchan], Hz                        */
+    const double *freq;         /* device f64 [nchan], Hz; also holds any channel
+                                 * that chan_of_vis names from nchan on          */
     const uint8_t *pa_bin;      /* device [nrow] or NULL (all 0)                 */
     const uint8_t *fbin;        /* device [nchan] or NULL (all 0)                */
     const uint8_t *flags;       /* device [nvis] or NULL; nonzero = flagged      */

@@ -14,7 +14,8 @@ struct CoordArgs {
     const double *uvw;
     const uint32_t *row;
     const uint16_t *chan;
-    const double *fl;          // per channel: frequency / c, one correctly rounded division
+    const double *freq;
+    const double *fl;          // channels [0, nchan): frequency / c, one correctly rounded division
     const uint8_t *pa_bin;
     const uint8_t *fbin;
     const uint8_t *flags;
@@ -46,13 +47,14 @@ __global__ void channel_kernel(const double *freq, int nchan, double *fl) {
 
 // The FP64 coordinate step with a fixed operation order (no contraction).
 // FP64 runs at 2 lanes a clock and SM here, so the step holds ten FP64 operations
-// and three conversions; the division by c is done once a channel, signs are
+// and three conversions; the division by c is done once a channel (a channel that
+// the descriptor's nchan does not count takes the same division here), signs are
 // tested and changed on the bits.
 __device__ __forceinline__ CoordOut coord_of(const CoordArgs &a, int64_t k) {
     CoordOut o;
     const uint32_t r = a.row[k];
     const uint16_t c = a.chan[k];
-    const double f = __ldg(a.fl + c);
+    const double f = (int)c < a.nchan ? __ldg(a.fl + c) : __ddiv_rn(a.freq[c], AW_C_LIGHT);
     double u = __dmul_rn(a.uvw[3 * (int64_t)r + 0], f);
     double v = __dmul_rn(a.uvw[3 * (int64_t)r + 1], f);
     double w = __dmul_rn(a.uvw[3 * (int64_t)r + 2], f);
@@ -492,6 +494,7 @@ int fill_coord_args(const aw_vis_desc *vis, const aw_kernel_set *ks, int tile, C
     a.uvw = vis->uvw;
     a.row = vis->row_of_vis;
     a.chan = vis->chan_of_vis;
+    a.freq = vis->freq;
     a.fl = plan->d_fl;
     a.pa_bin = vis->pa_bin;
     a.fbin = vis->fbin;
@@ -828,10 +831,10 @@ int aw_plan_build(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *ks, 
     std::vector<int32_t> sup(ks->supports.begin(), ks->supports.end());
     plan->bin_support = ks->bin_support;
     const int64_t n = vis->nvis;
-    const int nchan = std::max(vis->nchan, 1);
+    const int nchan = std::min(std::max(vis->nchan, 0), 65536);   // (chan_of_vis has 16 bits)
     const bool region = t.grid_mode == AW_GRID_REGION;
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_plane_support, sizeof(int32_t) * std::max<size_t>(sup.size(), 1)));
-    AW_CUDA_TRY(aw_dev_malloc(&plan->d_fl, sizeof(double) * nchan));
+    AW_CUDA_TRY(aw_dev_malloc(&plan->d_fl, sizeof(double) * std::max(nchan, 1)));
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_wsum, sizeof(double)));
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_nonfinite, sizeof(unsigned long long)));
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_counter, sizeof(unsigned int) * (4 + AW_RG_COUNTERS)));
@@ -851,8 +854,8 @@ int aw_plan_build(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *ks, 
         AW_CUDA_TRY(cudaStreamSynchronize(s));
         return AW_OK;
     }
-    if (vis->nchan > 0) {
-        channel_kernel<<<grid_blocks(vis->nchan, 256), 256, 0, s>>>(vis->freq, vis->nchan, plan->d_fl);
+    if (nchan > 0) {
+        channel_kernel<<<grid_blocks(nchan, 256), 256, 0, s>>>(vis->freq, nchan, plan->d_fl);
         AW_CHECK_LAUNCH();
     }
     CoordArgs a;
@@ -960,6 +963,7 @@ int aw_plan_coords_impl(const aw_plan *plan, const aw_kernel_set *ks_unused, int
     a.uvw = vis->uvw;
     a.row = vis->row_of_vis;
     a.chan = vis->chan_of_vis;
+    a.freq = vis->freq;
     a.fl = plan->d_fl;
     a.pa_bin = vis->pa_bin;
     a.fbin = vis->fbin;
@@ -975,6 +979,7 @@ int aw_plan_coords_impl(const aw_plan *plan, const aw_kernel_set *ks_unused, int
     a.half = plan->half;
     a.winv = plan->winv;
     a.support = plan->d_plane_support;
+    a.nchan = vis->nchan;
     a.tile = plan->tune.tile;
     a.tbits = ilog2(plan->tune.tile);
     a.ntx = a.nty = (plan->N + plan->tune.tile - 1) / plan->tune.tile;

@@ -46,3 +46,30 @@ def test_orders(n, wide):
     cnt = np.unique(grp[ok], return_counts=True)[1]
     info = aw.aw_plan_query(plan)
     assert info.nitems_degrid == int(((cnt + 31) // 32).sum()) and info.nvalid == int(ok.sum())
+
+
+# a descriptor whose nchan does not count every channel in use (C callers may leave it
+# 0) gives the plan of the full one: the frequencies come from the caller's array
+@pytest.mark.parametrize("nchan", [-1, 0, 2])
+def test_channels_beyond_nchan(nchan):
+    from paper_2206_15117_gb300 import aw
+    ctx = aw.aw_create(0)
+    n = 5000
+    rng = np.random.default_rng(3)
+    dev = [torch.as_tensor(x, device="cuda") for x in
+           (rng.uniform(-1.0, 1.0, (200, 3)) * 50.0, rng.integers(0, 200, n).astype(np.int32),
+            rng.integers(0, 5, n).astype(np.int16), np.linspace(1.2e9, 1.5e9, 5))]
+    ks = aw.aw_make_kernels(ctx, N=256, dl=0.4 / 256, OS=4, npol=1, nw=2, w_max=260.0, supports=[8, 12])
+    got = []
+    for k in (5, nchan):
+        vd = aw.vis_desc(*dev)
+        vd.nchan = k
+        plan = aw.aw_plan_create(ctx, vd, ks, aw.aw_tune(32, 256, 2, 256, aw.AW_GRID_REGION))
+        out = {c: torch.empty(n, dtype=torch.int32, device="cuda") for c in ("x0", "y0", "fx", "fy", "bin")}
+        perm = torch.empty(n, dtype=torch.int32, device="cuda")
+        aw.aw_plan_coords(plan, **out)
+        aw.aw_plan_order(plan, perm)
+        got.append([x.cpu().numpy() for x in (*out.values(), perm)])
+        assert aw.aw_plan_query(plan).nvalid > 1000
+    for a, b in zip(*got):
+        np.testing.assert_array_equal(a, b)
