@@ -430,7 +430,10 @@ int aw_mosaic_combine(aw_ctx *ctx, const float *images, const float *beams, cons
     const int64_t npix = (int64_t)N * N;
     const uintptr_t at = (uintptr_t)images | (uintptr_t)beams | (uintptr_t)gamma | (uintptr_t)out;
     auto apart = [&](const float *p, int64_t n) { return out + (int64_t)nplane * npix <= p || out >= p + n; };
-    if (npix % 4 == 0 && at % 16 == 0 && apart(gamma, npix) && apart(beams, (int64_t)nfield * npix)) {
+    // the four-pixel form works on several planes of a pixel at a time, so an output over
+    // the images has to be theirs from the start; other overlaps take the planes in order
+    if (npix % 4 == 0 && at % 16 == 0 && apart(gamma, npix) && apart(beams, (int64_t)nfield * npix) &&
+        (out == images || apart(images, (int64_t)nfield * nplane * npix))) {
         const int64_t nq = npix / 4;
         combine4_kernel<<<(unsigned)((nq + 63) / 64), dim3(64, 4), 0, S_(stream)>>>(
             reinterpret_cast<const float4 *>(images), reinterpret_cast<const float4 *>(beams),

@@ -49,3 +49,23 @@ def test_combine_forms(ctx, N, off, nf, nplane):
     aw.aw_mosaic_combine(ctx, dev(imgs), dev(beams), dev(gam), out)
     ref = om.combine(imgs, beams, gam)
     assert np.abs(out.cpu().numpy() - ref).max() < 1e-5 * np.abs(ref).max()
+
+
+# an output that shares memory with the images: in place, and from one plane before
+# them on (a plane's output over the plane that has been read already)
+@pytest.mark.parametrize("before", [0, 1])
+@pytest.mark.parametrize("nplane", [4, 9])
+def test_combine_over_its_images(ctx, nplane, before):
+    from paper_2206_15117_gb300 import aw
+    N, nf = 256, 3
+    rng = np.random.default_rng(nplane)
+    imgs = rng.normal(size=(nf, nplane, N, N)).astype(np.float32)
+    beams = rng.uniform(0, 1, size=(nf, N, N)).astype(np.float32)
+    gam = oc.mosaic_gamma(beams.astype(np.float64), 0.1).astype(np.float32)
+    buf = torch.zeros((before + nf * nplane, N, N), dtype=torch.float32, device="cuda")
+    buf[before:] = torch.as_tensor(imgs.reshape(-1, N, N))
+    out = buf[:nplane]
+    aw.aw_mosaic_combine(ctx, buf[before:].view(nf, nplane, N, N), torch.as_tensor(beams, device="cuda"),
+                         torch.as_tensor(gam, device="cuda"), out)
+    ref = om.combine(imgs, beams, gam)
+    assert np.abs(out.cpu().numpy() - ref).max() < 1e-5 * np.abs(ref).max()
