@@ -230,6 +230,12 @@ inline bool aw_rg_eligible(int S, int npol) {
 __host__ __device__ inline int aw_rg_pack(int tx, int ty, int bx, int by) {
     return tx | ty << 9 | bx << 18 | by << 21;
 }
+// Whether 32-bit words hold the task positions and the queue head, which counts a
+// task once a plane and, at the end, once more for every CTA: a set of more tasks
+// (above a thousand million segments of one visibility or so) takes OFFSETS.
+inline bool aw_rg_fits(unsigned long long ntasks, int npol) {
+    return ntasks <= (0xffffffffull - (1ull << 20)) / (unsigned)npol;
+}
 
 // Visibilities per degridding work item: 8 warps x 4 visibilities.
 constexpr int AW_DG_VB = 4;

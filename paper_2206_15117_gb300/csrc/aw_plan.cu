@@ -395,14 +395,20 @@ __global__ void emit_items_kernel(const uint32_t *starts, const uint32_t *itemba
 
 // REGION tasks of the segments (one bin and one region tile each): ceil(count /
 // cap) pieces times blk^2 footprint blocks, geo[bin] = {tile side, cap, blk, -}.
+// *total: their number, in 64 bits (the positions in the list have 32).
 __global__ void rg_count_kernel(const uint32_t *starts, int64_t nseg, uint32_t nreg, const aw_rec *rec,
-                                const int4 *geo, uint32_t *ntask) {
+                                const int4 *geo, uint32_t *ntask, unsigned long long *total) {
+    unsigned long long sum = 0;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < nseg;
          s += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t a = starts[s], b = (s + 1 < nseg) ? starts[s + 1] : nreg;
         const int4 g = geo[rec[a].bin];
-        ntask[s] = (b - a + g.y - 1) / g.y * g.z * g.z;
+        const uint32_t n = (b - a + g.y - 1) / g.y * g.z * g.z;
+        ntask[s] = n;
+        sum += n;
     }
+    for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if ((threadIdx.x & 31) == 0 && sum) atomicAdd(total, sum);
 }
 
 __global__ void rg_emit_kernel(const uint32_t *starts, const uint32_t *base, int64_t nseg, uint32_t nreg,
@@ -624,16 +630,24 @@ int build_items(const K *keys, int64_t nv, int shift, int chunk, const aw_rec *r
 }
 
 // The region tasks of the nseg segments (b.words[2]) of the nreg records `rec`
-// under the per-bin geometry geo; allocates *tasks.
-int build_region_tasks(int64_t nseg, int64_t nreg, const aw_rec *rec, const int4 *geo, SortBufs &b, int4 **tasks,
-                       int64_t *ntasks, cudaStream_t s) {
-    rg_count_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>(b.words[2], nseg, (uint32_t)nreg, rec, geo, b.words[0]);
+// under the per-bin geometry geo; allocates *tasks.  *ntasks = 0 and no list if
+// they are more than aw_rg_fits allows.
+int build_region_tasks(int64_t nseg, int64_t nreg, int npol, const aw_rec *rec, const int4 *geo,
+                       unsigned long long *d_total, SortBufs &b, int4 **tasks, int64_t *ntasks, cudaStream_t s) {
+    unsigned long long total = 0;
+    *ntasks = 0;
+    AW_CUDA_TRY(cudaMemsetAsync(d_total, 0, sizeof(total), s));
+    rg_count_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>(b.words[2], nseg, (uint32_t)nreg, rec, geo, b.words[0], d_total);
     AW_CHECK_LAUNCH();
-    const int rc = scan_counts(b.words[0], b.words[1], nseg, b.scratch, ntasks, s);
+    const int rc = aw_exclusive_scan_u32(b.words[0], b.words[1], nseg, b.scratch, s);
     if (rc) return rc;
-    AW_CUDA_TRY(aw_dev_malloc(tasks, sizeof(int4) * std::max<int64_t>(*ntasks, 1)));
+    AW_CUDA_TRY(cudaMemcpyAsync(&total, d_total, sizeof(total), cudaMemcpyDeviceToHost, s));
+    AW_CUDA_TRY(cudaStreamSynchronize(s));
+    if (!aw_rg_fits(total, npol)) return AW_OK;
+    AW_CUDA_TRY(aw_dev_malloc(tasks, sizeof(int4) * std::max<int64_t>((int64_t)total, 1)));
     rg_emit_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>(b.words[2], b.words[1], nseg, (uint32_t)nreg, rec, geo, *tasks);
     AW_CHECK_LAUNCH();
+    *ntasks = (int64_t)total;
     return AW_OK;
 }
 
@@ -707,12 +721,18 @@ static int sort_region(aw_plan *plan, int64_t nv, const int4 *d_geo, int nb, int
         return AW_OK;
     }
     if (rc == AW_OK)
-        rc = build_region_tasks(nseg, plan->nreg, plan->d_rec_rg, d_geo, b, &plan->d_items_rg, &plan->nitems_rg, s);
+        rc = build_region_tasks(nseg, plan->nreg, plan->npol, plan->d_rec_rg, d_geo, d_nreg, b, &plan->d_items_rg,
+                                &plan->nitems_rg, s);
+    if (rc == AW_OK && plan->nitems_rg == 0) {   // too many tasks
+        plan->nreg = 0;
+        return AW_OK;
+    }
     // region degridding pays a region's load (and its latency) per task: for tasks that
     // are half full on average (20.16M Stokes-I visibilities, 237 a task: 2.7 against
     // 5.7 ms; 1M, 80 a task: 472 against 357 us)
     if (rc == AW_OK && plan->npol == 1 && plan->nreg >= (int64_t)RDG_MIN * nseg) {
-        rc = build_region_tasks(nseg, plan->nreg, plan->d_rec_rg, d_geo + nb, b, &plan->d_items_rgd, &plan->nitems_rgd, s);
+        rc = build_region_tasks(nseg, plan->nreg, 1, plan->d_rec_rg, d_geo + nb, d_nreg, b, &plan->d_items_rgd,
+                                &plan->nitems_rgd, s);
         if (rc == AW_OK && plan->nreg < (int64_t)RDG_MIN * plan->nitems_rgd) plan->nitems_rgd = 0;
     }
     return rc;
