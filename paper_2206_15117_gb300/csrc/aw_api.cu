@@ -224,7 +224,9 @@ int aw_kernel_set_destroy(aw_kernel_set *k) {
 static void free_plan(aw_plan *p) {
     if (!p) return;
     p->drop_graphs();
-    if (p->d_block) aw_dev_free(p->d_block);
+    if (p->d_rec) aw_dev_free(p->d_rec);
+    if (p->d_rec_dg) aw_dev_free(p->d_rec_dg);
+    if (p->d_rec_rg) aw_dev_free(p->d_rec_rg);
     if (p->d_plane_support) aw_dev_free(p->d_plane_support);
     if (p->d_fl) aw_dev_free(p->d_fl);
     if (p->d_wsum) aw_dev_free(p->d_wsum);

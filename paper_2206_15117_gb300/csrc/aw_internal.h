@@ -124,7 +124,6 @@ struct aw_plan {
     int ntype = 1;                  // baseline classes are ntype^2 when ntype >= 2
     aw_tune tune{};
     double mean_taps = 0;
-    void *d_block = nullptr;        // one allocation: d_rec, d_rec_dg, d_rec_rg
     aw_rec *d_rec = nullptr;        // [nvis] sorted (valid first) by (bin, tile, position)
     int4 *d_items = nullptr;        // [nitems] {start, count, bin, 0}
     // degridding order: the valid visibilities by (bin, super-tile, oversampled

@@ -525,16 +525,14 @@ int fill_coord_args(const aw_vis_desc *vis, const aw_kernel_set *ks, int tile, C
     return AW_OK;
 }
 
-// One device allocation handed out in pieces (buf: freed with the arena, for the
-// temporaries; else the plan frees it).
+// The temporaries: one device allocation handed out in pieces.
 struct Arena {
     DevBuf buf;
-    void *base = nullptr;
     size_t size = 0, used = 0;
     static size_t round(size_t b) { return (b + 255) / 256 * 256; }
     template <class T>
     T *take(size_t count) {
-        T *p = reinterpret_cast<T *>(static_cast<char *>(base) + used);
+        T *p = reinterpret_cast<T *>(static_cast<char *>(buf.p) + used);
         used += round(count * sizeof(T));
         return p;
     }
@@ -712,18 +710,22 @@ static int sort_region(aw_plan *plan, int64_t nv, const int4 *d_geo, int nb, int
     AW_CUDA_TRY(cudaStreamSynchronize(s));
     plan->nreg = (int64_t)nreg;
     if (plan->nreg == 0) return AW_OK;
-    gather_rec_kernel<<<grid_blocks(plan->nreg, 256), 256, 0, s>>>(plan->d_rec_dg, perm, plan->nreg, plan->d_rec_rg);
-    AW_CHECK_LAUNCH();
     int64_t nseg = 0;
     rc = build_segments<K>(keys, plan->nreg, 0, b, &nseg, s);
     if (rc == AW_OK && plan->npol == 4 && plan->nreg < RG_SPARSE * nseg) {
         plan->nreg = 0;
         return AW_OK;
     }
-    if (rc == AW_OK)
+    if (rc == AW_OK) {
+        AW_CUDA_TRY(aw_dev_malloc(&plan->d_rec_rg, sizeof(aw_rec) * plan->nreg));
+        gather_rec_kernel<<<grid_blocks(plan->nreg, 256), 256, 0, s>>>(plan->d_rec_dg, perm, plan->nreg, plan->d_rec_rg);
+        AW_CHECK_LAUNCH();
         rc = build_region_tasks(nseg, plan->nreg, plan->npol, plan->d_rec_rg, d_geo, d_nreg, b, &plan->d_items_rg,
                                 &plan->nitems_rg, s);
+    }
     if (rc == AW_OK && plan->nitems_rg == 0) {   // too many tasks
+        aw_dev_free(plan->d_rec_rg);
+        plan->d_rec_rg = nullptr;
         plan->nreg = 0;
         return AW_OK;
     }
@@ -745,7 +747,7 @@ static int build_region(aw_plan *plan, const aw_kernel_set *ks, int64_t nv, Sort
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // gridding geometry of every bin, then the degridding one
     std::vector<int4> geo((size_t)nb * 2, make_int4(0, 0, 0, 0));
-    bool all = true;
+    bool all = true, any = false;
     for (int i = 0; i < nb; ++i) {
         const int S = ks->bin_support[(size_t)i];
         if (ks->max_support > AW_RG_MIN_SUPPORT && aw_rg_eligible(S, plan->npol)) {
@@ -757,22 +759,26 @@ static int build_region(aw_plan *plan, const aw_kernel_set *ks, int64_t nv, Sort
             const int64_t capd = std::min<int64_t>(std::max<int64_t>(nv / (sms * 12) / 32 * 32, 32), AW_RG_MAXV_DG);
             geo[(size_t)i] = make_int4(aw_rg_tile(S), (int)cap, aw_rg_nblk(S), 0);
             geo[(size_t)nb + i] = make_int4(aw_rg_tile(S), (int)capd, 1, 0);
+            any = true;
         } else {
             all = false;
         }
     }
-    DevBuf dgeo, dcnt;
-    AW_CUDA_TRY(aw_dev_malloc(&dgeo.p, sizeof(int4) * geo.size()));
-    AW_CUDA_TRY(cudaMemcpyAsync(dgeo.p, geo.data(), sizeof(int4) * geo.size(), cudaMemcpyHostToDevice, s));
-    AW_CUDA_TRY(aw_dev_malloc(&dcnt.p, sizeof(unsigned long long)));
-    AW_CUDA_TRY(cudaMemsetAsync(dcnt.p, 0, sizeof(unsigned long long), s));
-    const int nt = (plan->N + aw_rg_tile(128) - 1) / aw_rg_tile(128);   // tiles an axis at the smallest tile side
-    const uint64_t maxkey = (uint64_t)nb * nt * nt;                     // also the key of the bins that take no region
-    const int4 *d_geo = (const int4 *)dgeo.p;
-    unsigned long long *d_nreg = (unsigned long long *)dcnt.p;
-    const int rc = key_bits(maxkey) <= 32 ? sort_region<uint32_t>(plan, nv, d_geo, nb, nt, maxkey, d_nreg, b, s)
-                                          : sort_region<uint64_t>(plan, nv, d_geo, nb, nt, maxkey, d_nreg, b, s);
-    if (rc) return rc;
+    if (any) {
+        DevBuf dgeo, dcnt;
+        AW_CUDA_TRY(aw_dev_malloc(&dgeo.p, sizeof(int4) * geo.size()));
+        AW_CUDA_TRY(cudaMemcpyAsync(dgeo.p, geo.data(), sizeof(int4) * geo.size(), cudaMemcpyHostToDevice, s));
+        AW_CUDA_TRY(aw_dev_malloc(&dcnt.p, sizeof(unsigned long long)));
+        AW_CUDA_TRY(cudaMemsetAsync(dcnt.p, 0, sizeof(unsigned long long), s));
+        const int nt = (plan->N + aw_rg_tile(128) - 1) / aw_rg_tile(128);   // tiles an axis at the smallest tile side
+        const uint64_t maxkey = (uint64_t)nb * nt * nt;                     // also the key of the bins that take no region
+        const int4 *d_geo = (const int4 *)dgeo.p;
+        unsigned long long *d_nreg = (unsigned long long *)dcnt.p;
+        const int rc = key_bits(maxkey) <= 32 ? sort_region<uint32_t>(plan, nv, d_geo, nb, nt, maxkey, d_nreg, b, s)
+                                              : sort_region<uint64_t>(plan, nv, d_geo, nb, nt, maxkey, d_nreg, b, s);
+        if (rc) return rc;
+        AW_CUDA_TRY(cudaStreamSynchronize(s));   // the geometry is freed here
+    }
     if (plan->nreg == 0) {
         all = false;
         std::fill(geo.begin(), geo.end(), make_int4(0, 0, 0, 0));
@@ -852,21 +858,13 @@ int aw_plan_build(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *ks, 
     plan->bin_support = ks->bin_support;
     const int64_t n = vis->nvis;
     const int nchan = std::min(std::max(vis->nchan, 0), 65536);   // (chan_of_vis has 16 bits)
-    const bool region = t.grid_mode == AW_GRID_REGION;
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_plane_support, sizeof(int32_t) * std::max<size_t>(sup.size(), 1)));
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_fl, sizeof(double) * std::max(nchan, 1)));
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_wsum, sizeof(double)));
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_nonfinite, sizeof(unsigned long long)));
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_counter, sizeof(unsigned int) * (4 + AW_RG_COUNTERS)));
     plan->d_rcounter = plan->d_counter + 4;
-    // the records of the plan's orders, in one allocation
-    Arena keep;
-    keep.size = (region ? 3 : 2) * Arena::round(sizeof(aw_rec) * std::max<int64_t>(n, 1));
-    AW_CUDA_TRY(aw_dev_malloc(&plan->d_block, keep.size));
-    keep.base = plan->d_block;
-    plan->d_rec = keep.take<aw_rec>(n);
-    plan->d_rec_dg = keep.take<aw_rec>(n);
-    if (region) plan->d_rec_rg = keep.take<aw_rec>(n);
+    AW_CUDA_TRY(aw_dev_malloc(&plan->d_rec, sizeof(aw_rec) * std::max<int64_t>(n, 1)));
     AW_CUDA_TRY(cudaMemcpyAsync(plan->d_plane_support, sup.data(), sizeof(int32_t) * sup.size(),
                                 cudaMemcpyHostToDevice, s));
     if (n == 0) {
@@ -895,7 +893,6 @@ int aw_plan_build(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *ks, 
               Arena::round(sizeof(aw_rec) * n) + 3 * Arena::round(sizeof(uint32_t) * words) +
               Arena::round(aw_scan_scratch_bytes((int64_t)words)) + Arena::round(sizeof(unsigned long long) * 4);
     AW_CUDA_TRY(aw_dev_malloc(&ar.buf.p, ar.size));
-    ar.base = ar.buf.p;
     SortBufs b;
     b.k0 = ar.take<uint64_t>(n);
     b.k1 = ar.take<uint64_t>(n);
@@ -954,6 +951,7 @@ int aw_plan_build(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *ks, 
         AW_CHECK_LAUNCH();
         int r = radix_sort<K>(keys, perm, nv, key_bits(ngroups), b, s);
         if (r) return r;
+        AW_CUDA_TRY(aw_dev_malloc(&plan->d_rec_dg, sizeof(aw_rec) * nv));
         gather_rec_kernel<<<grid_blocks(nv, 256), 256, 0, s>>>(plan->d_rec, perm, nv, plan->d_rec_dg);
         AW_CHECK_LAUNCH();
         return build_items<K>(keys, nv, 0, AW_DG_CHUNK, plan->d_rec_dg, b, &plan->d_items_dg, &plan->nitems_dg, s);

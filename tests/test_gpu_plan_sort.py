@@ -73,3 +73,34 @@ def test_channels_beyond_nchan(nchan):
         assert aw.aw_plan_query(plan).nvalid > 1000
     for a, b in zip(*got):
         np.testing.assert_array_equal(a, b)
+
+
+# what a REGION plan keeps beyond an OFFSETS plan where no bin takes a region (no support
+# with a region form; a sparse full-pol set): the OFFSETS items, no second order
+@pytest.mark.parametrize("kw", [dict(N=512, npol=1, nw=2, w_max=260.0, supports=[9, 17]),
+                                dict(N=512, npol=1, nw=1, supports=[7]),
+                                dict(N=4096, npol=4, nw=1, supports=[16], pa=[0.0, 0.1, 0.2, 0.3],
+                                     fbin_freqs=[1.2e9, 1.3e9, 1.4e9, 1.5e9])])
+def test_memory_without_regions(kw):
+    from paper_2206_15117_gb300 import aw
+    ctx = aw.aw_create(0)
+    n, nrow = 2000000, 100000
+    rng = np.random.default_rng(4)
+    half = 0.45 * kw["N"] / 0.4                     # 0.45 of the grid at the highest frequency
+    uvw = rng.uniform(-1.0, 1.0, (nrow, 3)) * (half * 299792458.0 / 1.5e9, half * 299792458.0 / 1.5e9, 50.0)
+    pa, fb = rng.integers(0, 4, nrow).astype(np.uint8), rng.integers(0, 4, 16).astype(np.uint8)
+    dev = [torch.as_tensor(x, device="cuda") for x in
+           (uvw, rng.integers(0, nrow, n).astype(np.int32), rng.integers(0, 16, n).astype(np.int16),
+            np.linspace(1.2e9, 1.5e9, 16), pa, fb)]
+    ks = aw.aw_make_kernels(ctx, **kw, dl=0.4 / kw["N"], OS=4)
+    vd = aw.vis_desc(*dev)
+
+    def kept(mode):
+        aw.aw_plan_destroy(aw.aw_plan_create(ctx, vd, ks, aw.aw_tune(32, 256, 2, 1024, mode)))
+        free = torch.cuda.mem_get_info()[0]
+        plan = aw.aw_plan_create(ctx, vd, ks, aw.aw_tune(32, 256, 2, 1024, mode))
+        info = aw.aw_plan_query(plan)
+        assert info.region_lists == 0 and info.nvalid > n // 2
+        return free - torch.cuda.mem_get_info()[0], info.nitems_degrid
+    (offsets, items), (region, _) = kept(aw.AW_GRID_OFFSETS), kept(aw.AW_GRID_REGION)
+    assert region <= offsets + 16 * items + (4 << 20), (region, offsets, items)   # (two allocations' rounding)
