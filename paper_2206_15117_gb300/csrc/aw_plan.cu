@@ -629,8 +629,9 @@ int build_items(const K *keys, int64_t nv, int shift, int chunk, const aw_rec *r
 
 // The region tasks of the nseg segments (b.words[2]) of the nreg records `rec`
 // under the per-bin geometry geo; allocates *tasks.  *ntasks = 0 and no list if
-// they are more than aw_rg_fits allows.
-int build_region_tasks(int64_t nseg, int64_t nreg, int npol, const aw_rec *rec, const int4 *geo,
+// they are more than aw_rg_fits allows or hold fewer than min_mean visibilities on
+// average.
+int build_region_tasks(int64_t nseg, int64_t nreg, int npol, int64_t min_mean, const aw_rec *rec, const int4 *geo,
                        unsigned long long *d_total, SortBufs &b, int4 **tasks, int64_t *ntasks, cudaStream_t s) {
     unsigned long long total = 0;
     *ntasks = 0;
@@ -641,7 +642,7 @@ int build_region_tasks(int64_t nseg, int64_t nreg, int npol, const aw_rec *rec, 
     if (rc) return rc;
     AW_CUDA_TRY(cudaMemcpyAsync(&total, d_total, sizeof(total), cudaMemcpyDeviceToHost, s));
     AW_CUDA_TRY(cudaStreamSynchronize(s));
-    if (!aw_rg_fits(total, npol)) return AW_OK;
+    if (!aw_rg_fits(total, npol) || nreg < min_mean * (int64_t)total) return AW_OK;
     AW_CUDA_TRY(aw_dev_malloc(tasks, sizeof(int4) * std::max<int64_t>((int64_t)total, 1)));
     rg_emit_kernel<<<grid_blocks(nseg, 256), 256, 0, s>>>(b.words[2], b.words[1], nseg, (uint32_t)nreg, rec, geo, *tasks);
     AW_CHECK_LAUNCH();
@@ -682,20 +683,15 @@ static int build_hybrid_items(aw_plan *plan, cudaStream_t s) {
     return AW_OK;
 }
 
-// AW_GRID_REGION: the region order of the valid visibilities of the bins on
-// the region kernel, its tasks, and the OFFSETS items of the other bins with
-// the second stream.  The region kernel is the faster one at every support it
-// takes (aw_rg_eligible), so every plane goes there, split_planes or not.
-#ifndef RDG_MIN
-#define RDG_MIN 128
-#endif
+constexpr int64_t RDG_MIN = 128;   // visibilities a region degridding task, on average
 // Sparse full-pol sets take OFFSETS alone: below RG_SPARSE visibilities a bin and
 // region tile, clearing and adding the four planes of a region costs more than
 // atomics (25k visibilities of 128 bins on 4096^2, 4 a tile: 506 us against 173; 45 sets of
 // 20k-2.9M: OFFSETS the faster one in all 26 below 28, equal about 60, up to 0.55 of
 // its speed above 200).
 constexpr int64_t RG_SPARSE = 24;
-// The sort buffers are the plan builder's (>= nv).
+// The region order of the eligible bins and its tasks; the sort buffers are the
+// plan builder's (>= nv).
 template <typename K>
 static int sort_region(aw_plan *plan, int64_t nv, const int4 *d_geo, int nb, int nt, uint64_t maxkey,
                        unsigned long long *d_nreg, SortBufs &b, cudaStream_t s) {
@@ -720,7 +716,7 @@ static int sort_region(aw_plan *plan, int64_t nv, const int4 *d_geo, int nb, int
         AW_CUDA_TRY(aw_dev_malloc(&plan->d_rec_rg, sizeof(aw_rec) * plan->nreg));
         gather_rec_kernel<<<grid_blocks(plan->nreg, 256), 256, 0, s>>>(plan->d_rec_dg, perm, plan->nreg, plan->d_rec_rg);
         AW_CHECK_LAUNCH();
-        rc = build_region_tasks(nseg, plan->nreg, plan->npol, plan->d_rec_rg, d_geo, d_nreg, b, &plan->d_items_rg,
+        rc = build_region_tasks(nseg, plan->nreg, plan->npol, 0, plan->d_rec_rg, d_geo, d_nreg, b, &plan->d_items_rg,
                                 &plan->nitems_rg, s);
     }
     if (rc == AW_OK && plan->nitems_rg == 0) {   // too many tasks
@@ -729,17 +725,21 @@ static int sort_region(aw_plan *plan, int64_t nv, const int4 *d_geo, int nb, int
         plan->nreg = 0;
         return AW_OK;
     }
-    // region degridding pays a region's load (and its latency) per task: for tasks that
-    // are half full on average (20.16M Stokes-I visibilities, 237 a task: 2.7 against
-    // 5.7 ms; 1M, 80 a task: 472 against 357 us)
-    if (rc == AW_OK && plan->npol == 1 && plan->nreg >= (int64_t)RDG_MIN * nseg) {
-        rc = build_region_tasks(nseg, plan->nreg, 1, plan->d_rec_rg, d_geo + nb, d_nreg, b, &plan->d_items_rgd,
+    // Region degridding pays a region's load (and its latency) per task: taken where the
+    // tasks, as they are cut for this set, are half full on average (20.16M Stokes-I
+    // visibilities, 237 a task: 2.7 against 5.7 ms; 1M, 80 a task: 472 against 357 us).
+    // Their size is limited by the set's as well as by the tiles' density, so sets below
+    // RDG_MIN x 12 tasks an SM (233,000 visibilities on 152 SMs) never take it.
+    if (rc == AW_OK && plan->npol == 1 && plan->nreg >= RDG_MIN * nseg)
+        rc = build_region_tasks(nseg, plan->nreg, 1, RDG_MIN, plan->d_rec_rg, d_geo + nb, d_nreg, b, &plan->d_items_rgd,
                                 &plan->nitems_rgd, s);
-        if (rc == AW_OK && plan->nreg < (int64_t)RDG_MIN * plan->nitems_rgd) plan->nitems_rgd = 0;
-    }
     return rc;
 }
 
+// AW_GRID_REGION: the region order of the valid visibilities of the bins on
+// the region kernel, its tasks, and the OFFSETS items of the other bins with
+// the second stream.  The region kernel is the faster one at every support it
+// takes (aw_rg_eligible), so every plane goes there, split_planes or not.
 static int build_region(aw_plan *plan, const aw_kernel_set *ks, int64_t nv, SortBufs &b, cudaStream_t s) {
     const int nb = ks->nbins;
     int dev = 0, sms = 152;

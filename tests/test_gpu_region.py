@@ -94,3 +94,19 @@ def test_sparse_set_takes_offsets(ctx):
     _check_grid(c)
     _check_grid(c, batched=True)
     _check_degrid(c)
+
+
+# dense Stokes-I sets whose degridding tasks are too short for the region kernel keep no
+# list of them: as many device buffers as a sparse set's plan
+def test_short_degridding_tasks_are_not_kept(ctx):
+    from paper_2206_15117_gb300 import aw
+
+    def buffers(n_t, radius):
+        ob, kw = _stokes_i((16, 24, 40), n_t=n_t, radius=radius)
+        ks = aw.aw_make_kernels(ctx, **kw)
+        vd, keep = aw.device_observation(ob)
+        live = aw.aw_debug_alloc_stats()[0]
+        plan = aw.aw_plan_create(ctx, vd, ks, aw.aw_tune(32, 256, 2, 256, REGION))
+        assert aw.aw_plan_query(plan).region_lists > 0
+        return aw.aw_debug_alloc_stats()[0] - live
+    assert buffers(700, 20.0) == buffers(20, 120.0)
