@@ -780,10 +780,18 @@ int aw_debug_alloc_stats(int64_t *live, int64_t *calls);
  * code of the first failed check since the last reset, 0 if none (1-4 tile
  * gridding: grid, table, shared memory, record; 5-8 the same for the offset
  * schedule; 9-13 degridding: table source, shared-memory destination, grid,
- * partial sums, record); reset != 0 clears it.  Synchronises the device.
+ * partial sums, record; 14-18 region gridding: record, region cell, table, grid,
+ * shared memory; 19-22 region degridding: record, region cell, table, shared
+ * memory); reset != 0 clears it.  Synchronises the device.
  * AW_EUNSUPPORTED in a normal build.
  */
 int aw_debug_bounds_status(uint32_t *status, int32_t reset);
+/*
+ * aw_debug_region_tasks - tasks of the plan's region kernels: *grid of the
+ * gridding kernel (a task is done once per polarisation plane), *degrid of the
+ * Stokes-I degridding kernel; 0 where the plan does not launch that kernel.
+ */
+int aw_debug_region_tasks(const aw_plan *plan, int64_t *grid, int64_t *degrid);
 int aw_debug_wait_timeout(aw_ctx *ctx, int32_t which, void *stream);
 
 #ifdef __cplusplus

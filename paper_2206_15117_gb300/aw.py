@@ -119,6 +119,7 @@ SIGNATURES = {
     "aw_debug_alloc_stats": (ctypes.c_int, [ctypes.POINTER(c_i64), ctypes.POINTER(c_i64)]),
     "aw_debug_wait_timeout": (ctypes.c_int, [c_p, c_i32, c_p]),
     "aw_debug_bounds_status": (ctypes.c_int, [ctypes.POINTER(ctypes.c_uint32), c_i32]),
+    "aw_debug_region_tasks": (ctypes.c_int, [c_p, ctypes.POINTER(c_i64), ctypes.POINTER(c_i64)]),
     "aw_degrid_learned": (ctypes.c_int, [c_p, c_p, c_p, c_p, c_p, c_p, c_p]),
     "aw_surrogate_save": (ctypes.c_int, [c_p, ctypes.c_char_p]),
     "aw_kernel_spec_hash": (ctypes.c_int, [ctypes.POINTER(aw_kernel_spec), ctypes.POINTER(ctypes.c_uint64)]),
@@ -654,3 +655,10 @@ def aw_debug_bounds_status(reset: bool = False) -> int:
     st = ctypes.c_uint32()
     _check(load().aw_debug_bounds_status(ctypes.byref(st), int(bool(reset))), "aw_debug_bounds_status")
     return st.value
+
+
+def aw_debug_region_tasks(plan: Handle):
+    """(gridding tasks, degridding tasks) of the plan's region kernels."""
+    g, d = c_i64(0), c_i64(0)
+    _check(load().aw_debug_region_tasks(plan.ptr, ctypes.byref(g), ctypes.byref(d)), "aw_debug_region_tasks")
+    return int(g.value), int(d.value)

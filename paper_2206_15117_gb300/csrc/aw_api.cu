@@ -656,6 +656,13 @@ extern "C" int aw_debug_alloc_stats(int64_t *live, int64_t *calls) {
     return AW_OK;
 }
 
+extern "C" int aw_debug_region_tasks(const aw_plan *p, int64_t *grid, int64_t *degrid) {
+    if (!p || !grid || !degrid) return aw_set_error(AW_EINVAL, "NULL argument");
+    *grid = p->nitems_rg;
+    *degrid = p->nitems_rgd;
+    return AW_OK;
+}
+
 extern "C" int aw_debug_wait_timeout(aw_ctx *ctx, int32_t which, void *stream) {
     AW_GUARD_BEGIN
     if (!ctx) return aw_set_error(AW_EINVAL, "ctx is NULL");
