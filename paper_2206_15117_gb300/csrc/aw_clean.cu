@@ -39,8 +39,8 @@ constexpr int SCR_PEAK = 6;      // window peak |I| (float bits, >= 0)
 constexpr int SCR_NITER = 7;     // Hogbom iterations
 constexpr int SCR_BAR_COUNT = 8; // grid barrier: arrivals
 constexpr int SCR_BAR_ERR = 10;  // grid barrier: set when a wait gave up
-// spin limit of one barrier wait: 2^24 polls, about 9 s on GB300
-constexpr long long BAR_SPIN_LIMIT = 1ll << 24;
+// spin limit of one barrier wait: polls of 0.37 to 0.39 us (2^24 of them 6.2 s, 3 x 2^23 9.7 s), about 9 s
+constexpr long long BAR_SPIN_LIMIT = 24000000ll;
 
 // ---------------------------------------------------------------- sidelobe
 // r0 = first x > 0 with psf[c][c + x] <= 0 (N/2 if none), one warp.

@@ -96,3 +96,11 @@ def test_bounded_waits_give_up_and_the_context_stays_usable(ctx, which):
     assert st.n_gridded == aw.aw_plan_query(plan).nvalid > 0
     assert torch.isfinite(torch.view_as_real(grid)).all()
     assert aw.aw_debug_wait_timeout(ctx, 2) == aw.AW_EINVAL
+
+
+def test_barrier_wait_is_as_long_as_stated(ctx):
+    # about 9 s: a poll takes 0.37 us, and its share of fixed back-off does not scale with the clock
+    from paper_2206_15117_gb300 import aw
+    t0 = time.perf_counter()
+    assert aw.aw_debug_wait_timeout(ctx, 0) == aw.AW_ETIMEOUT
+    assert 7.5 < time.perf_counter() - t0 < 20.0
