@@ -155,7 +155,8 @@ typedef struct aw_tune {
                               * AW_GRID_REGION                                    */
     int32_t split_planes;    /* AW_GRID_HYBRID: visibilities in w planes
                               * [0, split_planes) take the TILES schedule, the
-                              * rest OFFSETS; 0..nw.  Ignored by the other modes */
+                              * rest OFFSETS; 0..nw.  AW_GRID_REGION: the same
+                              * range, no effect.  Ignored by the other modes     */
 } aw_tune;
 
 /* Gridding schedules (aw_tune.grid_mode).  TILES: work items of one bin and
@@ -177,10 +178,10 @@ typedef struct aw_tune {
  * support has no region form (padded to a multiple of 8 taps a side it would
  * cost more than 1.8 times the taps; Stokes I: above 48 cells; every support 8 or
  * less) take OFFSETS on the plan's second stream at the same time, and a full-pol
- * set with fewer than 24 visibilities a bin and region tile takes OFFSETS alone.  split_planes is checked (0..nw)
- * but does not move planes to OFFSETS, which is the slower one at every
- * support with a region form.  All modes give the same grid up to FP32
- * rounding order. */
+ * set with fewer than 24 visibilities a bin and region tile takes OFFSETS alone.
+ * split_planes is checked (0..nw) but does not move planes to OFFSETS, which is
+ * the slower one at every support with a region form.  All modes give the same
+ * grid up to FP32 rounding order. */
 enum { AW_GRID_TILES = 0, AW_GRID_OFFSETS = 1, AW_GRID_HYBRID = 2, AW_GRID_REGION = 3 };
 
 typedef struct aw_plan_info {
@@ -364,12 +365,12 @@ int aw_grid_batched(aw_ctx *ctx, aw_plan *plan, const aw_kernel_set *kset, const
 /*
  * aw_autotune - time aw_grid_batched over candidate (tile, chunk,
  * ctas_per_sm) of the TILES schedule, two super-tile sizes of the OFFSETS
- * schedule and up to three split planes (the first planes holding about 25,
- * 35 and 45 % of the visibility-taps) at 2 or 3 TILES CTAs per SM of the
- * HYBRID schedule on the given visibilities (pass a subsample to keep it
- * short) and return the fastest in *out; it is also kept in the context as the tune
- * aw_plan_create uses when given NULL.  Uses a scratch grid it allocates.
- * Synchronises `stream`.
+ * schedule, the REGION schedule (if a support has a region form) and up to
+ * three split planes (the first planes holding about 25, 35 and 45 % of the
+ * visibility-taps) at 2 or 3 TILES CTAs per SM of the HYBRID schedule on the
+ * given visibilities (pass a subsample to keep it short) and return the fastest
+ * in *out; it is also kept in the context as the tune aw_plan_create uses when
+ * given NULL.  Uses a scratch grid it allocates.  Synchronises `stream`.
  */
 int aw_autotune(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *kset, aw_tune *out,
                 void *stream);
@@ -384,9 +385,8 @@ int aw_autotune(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *kset, 
  * real part, c(q) = psi(2 l_q / F) the taper (grid correction); row/column 0
  * are written as 0.  grid (device complex64 [npol][N][N], kset's N and npol)
  * is used as FFT scratch and left transformed (the plain unscaled inverse FFT);
- * image: device float
- * [npol][N][N].  FP32 complex: the library's own two-pass transform for N = 256
- * to 4096, cuFFT and a grid-correction kernel otherwise.
+ * image: device float [npol][N][N].  FP32 complex: the library's own two-pass
+ * transform for N = 256 to 4096, cuFFT and a grid-correction kernel otherwise.
  */
 int aw_fft_to_image(aw_ctx *ctx, const aw_kernel_set *kset, void *grid, double weight_sum,
                     float *image, void *stream);

@@ -357,7 +357,8 @@ static int launch_planned(aw_ctx *ctx, const aw_plan *p, const aw_kernel_set *k,
     if (p->tune.grid_mode == AW_GRID_REGION) {
         // the region tasks on the caller's stream; the bins that take no region
         // with the OFFSETS kernel on the second stream at the same time, one CTA
-        // per SM (it fits beside the region CTAs in registers and threads)
+        // per SM, launched first: eight region CTAs fill an SM's registers and
+        // shared memory, so fewer of them run there until it ends
         if (p->nitems_ho == 0) return aw_launch_grid_region(p, k, vis, weight, grid, s);
         if (p->nreg == 0) {   // no bin takes a region: OFFSETS alone, every SM
             aw_grid_launch Lo{p, k, vis, weight, grid, false, 0, s, AW_GRID_OFFSETS, p->d_items_ho, p->nitems_ho};

@@ -1059,7 +1059,7 @@ int aw_launch_degrid(const aw_plan *p, const aw_kernel_set *k, const void *grid,
     a.nvis = p->nvis;
     a.nvalid = p->nvalid;
     a.tail_end = p->nvis;
-    if (p->nitems_rgd > 0 && !(p->npol == 1 && k->max_support <= DGS_MAXS)) {
+    if (p->nitems_rgd > 0) {   // (no set of supports up to DGS_MAXS alone: AW_RG_MIN_SUPPORT)
         // region tasks (and the visibilities not gridded) first, the other bins here
         const int rc = aw_launch_degrid_region(p, k, grid, vis_out, s, sub_from);
         if (rc || p->nitems_ho == 0) return rc;

@@ -161,7 +161,7 @@ struct aw_plan {
     // a footprint in one task)
     int4 *d_items_rgd = nullptr;
     int64_t nitems_rgd = 0;
-    unsigned int *d_rcounter = nullptr;   // work-queue heads of the region kernels
+    unsigned int *d_rcounter = nullptr;   // work-queue head of the region gridding (behind d_counter)
     // coordinate inputs kept for aw_plan_coords
     aw_vis_desc vis{};
     double uscale = 0, half = 0, winv = 0;
@@ -193,7 +193,6 @@ struct aw_plan {
 constexpr int AW_RG_R = 56;
 constexpr int AW_RG_MAXV = 1024;      // visibilities per gridding task
 constexpr int AW_RG_MAXV_DG = 256;   // visibilities per degridding task
-constexpr int AW_RG_COUNTERS = 4;
 
 // blocks along an axis: n24 of 24 taps, then n16 of 16 (S <= 8: one of 8)
 __host__ __device__ inline int aw_rg_n24(int S) {

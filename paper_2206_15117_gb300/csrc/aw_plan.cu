@@ -862,7 +862,7 @@ int aw_plan_build(aw_ctx *ctx, const aw_vis_desc *vis, const aw_kernel_set *ks, 
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_fl, sizeof(double) * std::max(nchan, 1)));
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_wsum, sizeof(double)));
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_nonfinite, sizeof(unsigned long long)));
-    AW_CUDA_TRY(aw_dev_malloc(&plan->d_counter, sizeof(unsigned int) * (4 + AW_RG_COUNTERS)));
+    AW_CUDA_TRY(aw_dev_malloc(&plan->d_counter, sizeof(unsigned int) * 5));
     plan->d_rcounter = plan->d_counter + 4;
     AW_CUDA_TRY(aw_dev_malloc(&plan->d_rec, sizeof(aw_rec) * std::max<int64_t>(n, 1)));
     AW_CUDA_TRY(cudaMemcpyAsync(plan->d_plane_support, sup.data(), sizeof(int32_t) * sup.size(),
