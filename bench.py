@@ -1152,7 +1152,7 @@ def run_ours(args, rank, world, dist):
                                         hybrid_split(aw, plan, kw, share)))
         finalists.append(aw.aw_tune(tune.tile, tune.chunk, 2, 1024, aw.AW_GRID_REGION, kw["nw"]))
         key = lambda t_: (t_.grid_mode, t_.ctas_per_sm if t_.grid_mode != aw.AW_GRID_OFFSETS else 0,
-                          t_.split_planes if t_.grid_mode in (aw.AW_GRID_HYBRID, aw.AW_GRID_REGION) else 0,
+                          t_.split_planes if t_.grid_mode == aw.AW_GRID_HYBRID else 0,   # (moves no planes of REGION)
                           t_.dg_tile or 1024)
         seen = {key(tune)}
         for t_ in finalists:

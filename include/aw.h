@@ -156,7 +156,9 @@ typedef struct aw_tune {
     int32_t split_planes;    /* AW_GRID_HYBRID: visibilities in w planes
                               * [0, split_planes) take the TILES schedule, the
                               * rest OFFSETS; 0..nw.  AW_GRID_REGION: the same
-                              * range, no effect.  Ignored by the other modes     */
+                              * range; moves no planes, but a cached tune applies
+                              * to sets of at least so many.  Ignored by the
+                              * other modes                                       */
 } aw_tune;
 
 /* Gridding schedules (aw_tune.grid_mode).  TILES: work items of one bin and
@@ -180,8 +182,8 @@ typedef struct aw_tune {
  * less) take OFFSETS on the plan's second stream at the same time, and a full-pol
  * set with fewer than 24 visibilities a bin and region tile takes OFFSETS alone.
  * split_planes is checked (0..nw) but does not move planes to OFFSETS, which is
- * the slower one at every support with a region form.  All modes give the same
- * grid up to FP32 rounding order. */
+ * the slower one at every support with a region form once the tiles are dense.
+ * All modes give the same grid up to FP32 rounding order. */
 enum { AW_GRID_TILES = 0, AW_GRID_OFFSETS = 1, AW_GRID_HYBRID = 2, AW_GRID_REGION = 3 };
 
 typedef struct aw_plan_info {

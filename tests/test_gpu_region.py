@@ -111,3 +111,19 @@ def test_short_degridding_tasks_are_not_kept(ctx):
         return aw.aw_debug_alloc_stats()[0] - live
     # 31850 visibilities a bin and tile, 96 a task; 19 a bin and tile
     assert buffers(700, 20.0) == buffers(2, 200.0)
+
+
+# a region schedule found on one set is used on sets that have its planes of supports up to
+# 40, as before the schedule took every plane; sets of fewer planes take OFFSETS
+def test_cached_region_tune_on_fewer_planes(ctx):
+    from paper_2206_15117_gb300 import aw
+    own = aw.aw_create(0)
+    ob, kw = case_fullpol(supports=(16, 24, 48), n_t=2000, radius=50.0)
+    vd, keep = aw.device_observation(ob)
+    t = aw.aw_autotune(own, vd, aw.aw_make_kernels(own, **kw))
+    if t.grid_mode != REGION:
+        pytest.skip("another schedule was the fastest: %d" % t.grid_mode)
+    assert t.split_planes == 2
+    for supports, lists in (((16, 24), 1), ((16,), 0)):
+        few = dict(kw, nw=len(supports), supports=list(supports))
+        assert aw.aw_plan_query(aw.aw_plan_create(own, vd, aw.aw_make_kernels(own, **few))).region_lists == lists
