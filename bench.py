@@ -989,7 +989,8 @@ def learned_degrid(ctx, dev, args, kw, kw_fine, vd, obs, stream, timed, kmax, ch
 # ----------------------------------------------------------------------------- GPU arm
 def wproj_case(reps: int):
     """Configuration 2 for profiling: 20.16M Stokes-I visibilities, 2048^2, 32 w planes (supports 8-64),
-    OS 8, FP32 tables; the region schedule (the bench's choice for this configuration); one untimed grid + degrid, then `reps` timed ones."""
+    OS 8, FP32 tables; the region schedule (the bench's choice for this configuration); one untimed
+    grid + degrid, then `reps` timed ones."""
     import torch
     from paper_2206_15117_gb300 import aw
     from paper_2206_15117_gb300 import build as awbuild
@@ -1514,8 +1515,8 @@ TRAFFIC_PER_VIS = {"region": 146.5e6 / 1139896, "degrid_items_kernel": 96.5e6 / 
 def roofline_entry(kernel, achieved, peak, peak_src, flops, g_ms, d_ms, region, nvalid, subset):
     """The `roofline` object of the dominant step (gridding if g_ms >= d_ms).  `traffic` is the
     scaled one-bin-pair capture when it describes the kernel that runs: the degridder; the region
-    capture predates the present region kernel (one plane a CTA), so for the region
-    schedule `traffic` is null and the previous figure stands beside it, labelled.  Null at the
+    capture is of an earlier region kernel (the present one has one plane a CTA), so for the region
+    schedule `traffic` is null and that figure stands beside it, labelled.  Null at the
     subset scale and for the other schedules."""
     traffic, traffic_prev = None, None
     if not subset:
@@ -1531,8 +1532,8 @@ def roofline_entry(kernel, achieved, peak, peak_src, flops, g_ms, d_ms, region, 
     if traffic_prev:
         roof["traffic_previous_region_kernel"] = {
             "bytes": traffic_prev,
-            "source": "profiles/dram_traffic_fullpol_aw_1pair.md (the former region kernel, four planes a CTA), "
-                      "scaled by the visibility count (lower bound)"}
+            "source": "profiles/dram_traffic_fullpol_aw_1pair.md (an earlier region kernel: four planes a CTA, "
+                      "paired passes), scaled by the visibility count (lower bound)"}
     return roof
 
 

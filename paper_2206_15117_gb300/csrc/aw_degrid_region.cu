@@ -15,9 +15,9 @@
 //
 // What bounds it: the shared-memory pipe (8 bytes a visibility-tap) and, at the
 // small supports, the reductions.  20.16M visibilities at 2048^2, supports 8-64:
-// 2.76 ms (that pipe 74 % busy) against 5.71 ms reading the grid through L1, one
-// gather per tap (load latency).  128 threads and 6 CTAs an SM: 4 CTAs 3.60, 64
-// threads and 8 CTAs 3.72, 256 threads and 4 CTAs 3.06 ms.
+// 2.9 ms (that pipe 74 % busy) against 5.8 ms reading the grid through L1, one
+// gather per tap (load latency).  On a GPU where 128 threads and 6 CTAs an SM take
+// 2.76 ms: 4 CTAs 3.60, 64 threads and 8 CTAs 3.72, 256 threads and 4 CTAs 3.06 ms.
 #include <algorithm>
 
 #include "aw_internal.h"

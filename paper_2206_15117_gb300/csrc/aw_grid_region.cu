@@ -25,12 +25,12 @@
 // visibility-tap and plane plus the kernel loads of every run; at full
 // polarisation the FP32 pipe has the same limit of 0.5 clocks per
 // visibility-tap.  Measured on 12M full-pol visibilities at 4096^2 (supports
-// 16-72): 24.9 ms (the pipe 79 % busy) against 34.3 ms for the former form, four
+// 16-72): 26.7 ms (the pipe 79 % busy) against 37.0 ms for the former form, four
 // planes a CTA with the warps kept apart by footprint-row residues and OFFSETS
-// beside it; 20.16M Stokes-I visibilities at 2048^2: 3.5 against 6.8 ms.  One
-// warp a region was slower (29.6 ms: two warps a scheduler do not hide their
-// own latencies), and so was loading the next run's kernel values into a second
-// register set (36-45 ms).
+// beside it; 20.16M Stokes-I visibilities at 2048^2: 3.9 against 7.4 ms.  On a GPU
+// where it takes 24.9 ms, one warp a region took 29.6 (two warps a scheduler do
+// not hide their own latencies) and loading the next run's kernel values into a
+// second register set 36-45 ms.
 #include <algorithm>
 
 #include "aw_internal.h"
@@ -162,8 +162,8 @@ struct Task {
 };
 
 // g + K V for the thread's taps.  Full polarisation in packed pairs (fma.rn.f32x2
-// runs at the FFMA rate with half the issue slots: 25.8 against 28.4 ms on the
-// set above): q1 = g + sum (kx, ky) vr, q2 = sum (kx, ky) vi, and g + K V =
+// runs at the FFMA rate with half the issue slots: 25.8 against 28.4 ms on that
+// GPU): q1 = g + sum (kx, ky) vr, q2 = sum (kx, ky) vi, and g + K V =
 // (q1.x - q2.y, q1.y + q2.x).
 template <int NPOL, int CB, int RB, bool PAD>
 __device__ __forceinline__ void add_vis(float2 *p, const float2 (&v)[NPOL], const float2 (&k)[CB * RB][NPOL],

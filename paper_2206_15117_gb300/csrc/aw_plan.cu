@@ -727,7 +727,7 @@ static int sort_region(aw_plan *plan, int64_t nv, const int4 *d_geo, int nb, int
     }
     // Region degridding pays a region's load (and its latency) per task: taken where the
     // tasks, as they are cut for this set, are half full on average (20.16M Stokes-I
-    // visibilities, 237 a task: 2.7 against 5.7 ms; 1M, 80 a task: 472 against 357 us).
+    // visibilities, 237 a task: 2.9 against 5.8 ms; 1M, 80 a task: 472 against 357 us).
     // Their size is limited by the set's as well as by the tiles' density, so sets below
     // RDG_MIN x 12 tasks an SM (233,000 visibilities on 152 SMs) never take it.
     if (rc == AW_OK && plan->npol == 1 && plan->nreg >= RDG_MIN * nseg)
